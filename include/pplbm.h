@@ -221,8 +221,8 @@ lbm_status lbm_save_state(lbm_ctx* ctx, void* host_buf, size_t bytes);
 lbm_status lbm_load_state(lbm_ctx* ctx, const void* host_buf, size_t bytes);
 
 /* Tile shape of the fused kernel: columns per CTA (64, 128 or 256; a CTA writes
- * cols - 8 columns, the other 8 cover halo columns; the scalar kernel runs cols
- * threads, the paired kernel cols / 2) and rows per CTA (>= 4, or the full height).
+ * cols - 8 columns, the other 8 cover halo columns; the one-column kernels run cols
+ * threads, the FP32 strip kernel 1, 2 or 5 warps) and rows per CTA (>= 4, or the full height).
  * Results do not depend on the shape except through the per-CTA sums of the
  * domain-mean density (Eq. 14) and their rounding to the fixed-point totals; only speed differs.  0 = default: the band plan of
  * lbm_default_band_plan for the CTA slots of the current device and kernel form. */
@@ -258,28 +258,28 @@ lbm_status lbm_default_band_plan(int32_t nx, int32_t ny, int32_t cols, int64_t s
 
 /* Form of the FP32 step kernel.  All forms compute the same step (Sec. 2; boundary
  * conditions of Sec. 2.C) and agree to FP32 rounding.
- *   LBM_KERNEL_SCALAR (and LBM_KERNEL_AUTO, the default): one column per thread; each
- *     thread stages the populations it pulls with per-element asynchronous copies
- *     (cp.async).  Handles every option.  The fastest form on GB300.
- *   LBM_KERNEL_PAIRED: each thread updates two adjacent columns with packed FP32
- *     arithmetic (two nodes per add / multiply / fused multiply-add) and 8-byte stores;
- *     about 40 % fewer instructions per node but fewer warps per SM, slower on GB300.
- *     Lattices with the Hazi-Markus source take the scalar form.
+ *   LBM_KERNEL_AUTO (the default), LBM_KERNEL_INTERIOR and LBM_KERNEL_PAIRED: one warp per strip
+ *     of at most 60 columns, two adjacent columns per lane with packed FP32 arithmetic (two nodes
+ *     per add / multiply / fused multiply-add), neighbours by shuffles, no barrier per row.
+ *     Handles every option; the fastest form on GB300.
+ *   LBM_KERNEL_SCALAR: one column per thread; each thread stages the populations it pulls with
+ *     per-element asynchronous copies (cp.async).  Handles every option.
  *   LBM_KERNEL_TMA: one column per thread; one thread per CTA stages whole rows of
  *     every population plane with bulk tensor copies (cp.async.bulk.tensor, completion
  *     on mbarriers), which removes the per-thread copy work from the step.  Needs
  *     128-column tiles and the step's lean form (no pool geometry, Hazi-Markus source
  *     or bubble statistics); other lattices take the scalar form.  A bulk copy that does
  *     not complete within a bounded wait (lbm_set_wait_limit) makes lbm_sync return
- *     LBM_ETIMEOUT.  Its results
- *     are bit-identical to the scalar form's; on GB300 it runs about 9 % slower (its
- *     warps wait on rows that arrive later than the per-thread copies do).
- * FP64 lattices, and lbm_step_noalloc on caller-laid-out buffers, always use the scalar
- * form.  LBM_EINVAL for other values. */
+ *     LBM_ETIMEOUT.  Its results are bit-identical to the scalar form's.
+ * FP64 lattices take the one-column kernel, with a path without per-node boundary logic for the
+ * tiles away from open ends and wraps unless LBM_KERNEL_SCALAR is asked for; lbm_step_noalloc on
+ * caller-laid-out buffers always uses the scalar form.  LBM_EINVAL for other values. */
 enum { LBM_KERNEL_AUTO = 0, LBM_KERNEL_SCALAR = 1, LBM_KERNEL_PAIRED = 2, LBM_KERNEL_TMA = 3, LBM_KERNEL_INTERIOR = 4 };
 lbm_status lbm_set_kernel(lbm_ctx* ctx, int32_t kernel);
-/* The form (LBM_KERNEL_SCALAR, _PAIRED or _TMA) the context's step launches take
- * with its current kernel request, precision, parameters and tiling; -1 if ctx is NULL. */
+/* The form (LBM_KERNEL_SCALAR, _INTERIOR, _PAIRED or _TMA) the context's step launches go by
+ * with its current kernel request, precision, parameters and tiling (_SCALAR where the pool
+ * geometry, the Hazi-Markus source or the bubble statistics need the per-node boundary logic,
+ * whichever kernel runs it); -1 if ctx is NULL. */
 int32_t lbm_step_kernel(const lbm_ctx* ctx);
 
 /* How lbm_step / lbm_step_async advance the lattice (a calling convention of the library;
@@ -301,8 +301,8 @@ int32_t lbm_step_kernel(const lbm_ctx* ctx);
  *     than the poll limit of lbm_set_wait_limit) gives up, the launch ends, and the next
  *     lbm_sync returns LBM_ETIMEOUT; the lattice state is then undefined until it is
  *     initialised again (lbm_set_params, lbm_init_fields, lbm_set_populations or
- *     lbm_load_state), and the CUDA context stays usable.  Only the one-column step forms
- *     (LBM_KERNEL_SCALAR, LBM_KERNEL_INTERIOR) have a persistent form.
+ *     lbm_load_state), and the CUDA context stays usable.  All forms but
+ *     LBM_KERNEL_TMA have a persistent form.
  *   LBM_LOOP_AUTO (default): persistent where the step tiling fits in one wave of the
  *     persistent kernel (small lattices, whose steps are short enough for the launch gap and
  *     the kernel boundary to count) or where it takes at least two and a half waves and the

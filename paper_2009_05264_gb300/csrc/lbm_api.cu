@@ -19,6 +19,10 @@ namespace pplbm {
 cudaError_t launch_lbm_f32(int, int, int, int, bool, const Inst*, const Tile*, int, cudaStream_t, const Inst*,
                           unsigned);
 cudaError_t launch_lbm_f64(int, int, int, int, bool, const Inst*, const Tile*, int, cudaStream_t, const Inst*);
+cudaError_t launch_strip(int, int, int, const Inst*, const Tile*, int, cudaStream_t, const Inst*);
+cudaError_t launch_strip_persistent(int, int, int, const Inst*, const Tile*, int, int, GridBar*, unsigned,
+                                    cudaStream_t, const Inst*, const FlowPlan&);
+int strip_resident_ctas(int, int, int, bool, bool);
 cudaError_t launch_init_from_fields_f32(const Inst*, int, int, const double*, int, cudaStream_t);
 cudaError_t launch_init_from_fields_f64(const Inst*, int, int, const double*, int, cudaStream_t);
 cudaError_t launch_init_builtin_f32(const Inst*, int, int, InitSpec, cudaStream_t);
@@ -31,25 +35,37 @@ cudaError_t launch_persistent_f64(int, int, int, bool, const Inst*, const Tile*,
 int persistent_resident_f32(int, int, int, bool, bool);
 int persistent_resident_f64(int, int, int, bool, bool);
 
-cudaError_t launch_persistent(int fp64, int thermal, int cols, int kernel, bool full, const Inst* d_inst,
+cudaError_t launch_persistent(int fp64, int thermal, int cols, int kernel, int flags, const Inst* d_inst,
                               const Tile* d_tiles, int ntiles, int nsteps, GridBar* bar, unsigned max_polls,
                               cudaStream_t s, const Inst* h_inst, const FlowPlan& flow) {
+  const bool full = (flags & STEP_FULL) != 0;
+  if (kernel == FORM_STRIP)
+    return launch_strip_persistent(thermal, cols, flags, d_inst, d_tiles, ntiles, nsteps, bar, max_polls, s, h_inst, flow);
   return fp64 ? launch_persistent_f64(thermal, cols, kernel, full, d_inst, d_tiles, ntiles, nsteps, bar, max_polls, s,
                                       h_inst, flow)
               : launch_persistent_f32(thermal, cols, kernel, full, d_inst, d_tiles, ntiles, nsteps, bar, max_polls, s,
                                       h_inst, flow);
 }
 
-long long persistent_slots(int fp64, int thermal, int cols, int kernel, bool full, bool single) {
+long long persistent_slots(int fp64, int thermal, int cols, int kernel, int flags, bool single) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (kernel == FORM_STRIP) {
+    // a barrier per step up to 8 warps per SM, overlapped steps above
+    const int warps8 = cols <= 64 ? 8 : cols <= 128 ? 4 : 1;  // CTAs of 1, 2 and 5 warps
+    return (long long)sms * std::min(warps8, strip_resident_ctas(thermal, cols, flags, single, true));
+  }
+  const bool full = (flags & STEP_FULL) != 0;
   const int per_sm = fp64 ? persistent_resident_f64(thermal, cols, kernel, full, single)
                           : persistent_resident_f32(thermal, cols, kernel, full, single);
   return (long long)sms * per_sm;
 }
 
-cudaError_t launch_lbm(int fp64, int thermal, int cols, int mode, int kernel, bool full, const Inst* d_inst,
+cudaError_t launch_lbm(int fp64, int thermal, int cols, int mode, int kernel, int flags, const Inst* d_inst,
                        const Tile* d_tiles, int ntiles, cudaStream_t s, const Inst* h_inst, unsigned max_polls) {
+  const bool full = (flags & STEP_FULL) != 0;
+  if (mode == MODE_STEP && kernel == FORM_STRIP)
+    return launch_strip(thermal, cols, flags, d_inst, d_tiles, ntiles, s, h_inst);
   return fp64 ? launch_lbm_f64(thermal, cols, mode, kernel, full, d_inst, d_tiles, ntiles, s, h_inst)
               : launch_lbm_f32(thermal, cols, mode, kernel, full, d_inst, d_tiles, ntiles, s, h_inst, max_polls);
 }
@@ -195,6 +211,10 @@ const char* fill_inst(Inst& I, const lbm_params* p, int nx, int ny, int pitch, l
   I.rho_vapor = p->rho_vapor;
   I.source_model = p->source_model;
   I.bubble_stats = p->bubble_stats;
+  if (!fp64) {
+    fill_consts<float>(I.strip.C, I, I.rho_ref);
+    fill_pair_consts(I.strip.P, I);
+  }
   return nullptr;
 }
 
@@ -247,10 +267,10 @@ BandPlan default_band_plan(int nx, int ny, int cols, long long slots) {
   return best;
 }
 
-long long step_wave_slots(int fp64, int thermal, int cols, int kernel) {
+long long step_wave_slots(int fp64, int thermal, int cols, int kernel, int flags) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int per_sm = fp64 ? resident_ctas_f64(thermal, cols, kernel) : resident_ctas_f32(thermal, cols, kernel);
+  const int per_sm = fp64 ? resident_ctas_f64(thermal, cols, kernel) : resident_ctas_f32(thermal, cols, kernel, flags);
   return (long long)sms * (per_sm > 0 ? per_sm : 1);
 }
 }  // namespace pplbm
@@ -470,14 +490,14 @@ lbm_status set_tiling(lbm_ctx* c, int cols, const BandPlan& plan) {
 }
 
 int step_kernel(const lbm_ctx* c, int cols) {
-  return resolve_kernel(c->kernel, c->prec == LBM_FP64, needs_full_step(c->hinst),
-                        c->params.source_model == LBM_SOURCE_HAZI_MARKUS, c->have_tmaps, cols);
+  return resolve_kernel(c->kernel, c->prec == LBM_FP64, needs_full_step(c->hinst), c->have_tmaps, cols);
 }
 
 // Re-choose the default tiling for the current kernel, precision and thermal flag.
 lbm_status retile_default(lbm_ctx* c, int cols) {
   const long long slots =
-      step_wave_slots(c->prec == LBM_FP64, c->have_params ? c->thermal : 1, cols, step_kernel(c, cols));
+      step_wave_slots(c->prec == LBM_FP64, c->have_params ? c->thermal : 1, cols, step_kernel(c, cols),
+                      step_flags(c->hinst));
   const lbm_status s = set_tiling(c, cols, default_band_plan(c->nx, c->ny, cols, slots));
   if (s == LBM_OK) c->rows_default = true;
   return s;
@@ -494,7 +514,7 @@ bool flow_eligible(const lbm_ctx* c) {
 bool overlapped(lbm_ctx* c) {
   if (!flow_eligible(c)) return false;
   const long long slots = persistent_slots(c->prec == LBM_FP64, c->thermal, c->cols, step_kernel(c, c->cols),
-                                           needs_full_step(c->hinst), true);
+                                           step_flags(c->hinst), true);
   return c->ntiles_step > slots;
 }
 
@@ -507,10 +527,10 @@ bool overlapped(lbm_ctx* c) {
 bool use_persistent(lbm_ctx* c) {
   if (c->loop == LBM_LOOP_LAUNCHES) return false;
   const int kernel = step_kernel(c, c->cols);
-  if (kernel != LBM_KERNEL_SCALAR && kernel != LBM_KERNEL_INTERIOR) return false;
+  if (!has_persistent(kernel)) return false;
   if (c->loop == LBM_LOOP_PERSISTENT) return true;
   const long long slots = persistent_slots(c->prec == LBM_FP64, c->thermal, c->cols, kernel,
-                                           needs_full_step(c->hinst), true);
+                                           step_flags(c->hinst), true);
   return c->ntiles_step <= slots || (flow_eligible(c) && 2 * (long long)c->ntiles_step >= 5 * slots);
 }
 
@@ -518,7 +538,7 @@ lbm_status launch(lbm_ctx* c, int mode) {
   const bool step_tiles = mode == MODE_STEP;
   const int kernel = step_tiles ? step_kernel(c, c->cols) : LBM_KERNEL_SCALAR;
   cudaError_t e = launch_lbm(c->prec == LBM_FP64, c->thermal, step_tiles ? c->cols : kAuxCols, mode, kernel,
-                             needs_full_step(c->hinst), c->d_inst,
+                             step_flags(c->hinst), c->d_inst,
                              step_tiles ? c->d_tiles_step : c->d_tiles_aux,
                              step_tiles ? c->ntiles_step : c->ntiles_aux, c->stream, &c->hinst, c->max_polls);
   if (e != cudaSuccess) return cuda_fail(c, e, "kernel launch");
@@ -756,7 +776,7 @@ lbm_status lbm_step_async(lbm_ctx* c, int64_t nsteps) {
   DeviceGuard g(c->device);
   if (nsteps >= 2 && use_persistent(c)) {
     const int kernel = step_kernel(c, c->cols);
-    const bool full = needs_full_step(c->hinst);
+    const int flags = step_flags(c->hinst);
     GridBar* bar = reinterpret_cast<GridBar*>(c->base + c->L.off_bar);
     FlowPlan flow{};
     if (overlapped(c)) {
@@ -781,7 +801,7 @@ lbm_status lbm_step_async(lbm_ctx* c, int64_t nsteps) {
       if (flow.enabled)
         LBM_CUDA(c, cudaMemsetAsync(flow.cell_done, 0, (size_t)c->ntiles_step * sizeof(unsigned long long),
                                     c->stream));
-      cudaError_t e = launch_persistent(c->prec == LBM_FP64, c->thermal, c->cols, kernel, full, c->d_inst,
+      cudaError_t e = launch_persistent(c->prec == LBM_FP64, c->thermal, c->cols, kernel, flags, c->d_inst,
                                         c->d_tiles_step, c->ntiles_step, n, bar, c->max_polls, c->stream, &c->hinst,
                                         flow);
       if (e != cudaSuccess) return cuda_fail(c, e, "persistent kernel launch");
@@ -1029,7 +1049,11 @@ lbm_status lbm_set_kernel(lbm_ctx* c, int32_t kernel) {
   return retile_default(c, c->cols);
 }
 
-int32_t lbm_step_kernel(const lbm_ctx* c) { return c ? step_kernel(c, c->cols) : -1; }
+int32_t lbm_step_kernel(const lbm_ctx* c) {
+  if (!c) return -1;
+  return reported_kernel(c->kernel, step_kernel(c, c->cols), needs_full_step(c->hinst),
+                         c->params.source_model == LBM_SOURCE_HAZI_MARKUS);
+}
 
 lbm_status lbm_set_step_loop(lbm_ctx* c, int32_t loop) {
   if (!c) return LBM_EINVAL;

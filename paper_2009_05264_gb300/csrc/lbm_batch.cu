@@ -42,7 +42,7 @@ struct lbm_batch {
   int cols = 128, rows = 0;   // rows 0: each member's default band height
   int kernel = LBM_KERNEL_AUTO;         // requested step kernel form
   int launch_kernel = LBM_KERNEL_SCALAR; // the form the batch's launches take (resolve_kernel)
-  bool any_full = false;  // a member needs the step's full form (pool, Hazi-Markus, bubble statistics)
+  int flags = 0;  // STEP_*: what the members' steps need between them
   // device tables of the current membership
   Inst* d_insts = nullptr;
   Tile* d_tiles = nullptr;
@@ -96,8 +96,7 @@ BandPlan member_plan(const lbm_batch* b, int nx, int ny, long long slots, double
 lbm_status rebuild(lbm_batch* b) {
   std::vector<Inst> insts;
   std::vector<Tile> tiles;
-  bool any_hazi = false;  // a member uses the Hazi-Markus source (no paired form)
-  bool any_full = false;
+  int flags = 0;
   bool all_tmaps = true;  // every member has the tensor maps of the TMA kernel
   const int w = b->cols - 8;
   double total = 0.0;
@@ -105,12 +104,11 @@ lbm_status rebuild(lbm_batch* b) {
     if (!m.ctx) continue;
     total += (double)m.nx * m.ny;
     const Inst I = lbm_internal_inst(m.ctx);
-    any_hazi = any_hazi || I.source_model == LBM_SOURCE_HAZI_MARKUS;
-    any_full = any_full || needs_full_step(I);
+    flags |= step_flags(I);
     all_tmaps = all_tmaps && I.tmaps != nullptr;
   }
-  const int launch_kernel = resolve_kernel(b->kernel, b->prec == LBM_FP64, any_full, any_hazi, all_tmaps, b->cols);
-  const long long slots = step_wave_slots(b->prec == LBM_FP64, b->thermal, b->cols, launch_kernel);
+  const int launch_kernel = resolve_kernel(b->kernel, b->prec == LBM_FP64, (flags & STEP_FULL) != 0, all_tmaps, b->cols);
+  const long long slots = step_wave_slots(b->prec == LBM_FP64, b->thermal, b->cols, launch_kernel, flags);
   // every member's tall bands first, then every member's short bands (a member's tile
   // indices, which fix its partial-sum order, are those of the member alone)
   std::vector<Tile> shorts;
@@ -200,7 +198,7 @@ lbm_status rebuild(lbm_batch* b) {
   LBM_BCUDA(b, cudaStreamSynchronize(b->stream));
   b->ntiles = (int)tiles.size();
   b->launch_kernel = launch_kernel;
-  b->any_full = any_full;
+  b->flags = flags;
   drop_graph(b);
   b->dirty = false;
   return LBM_OK;
@@ -208,7 +206,7 @@ lbm_status rebuild(lbm_batch* b) {
 
 lbm_status launch_steps(lbm_batch* b, int64_t n) {
   for (int64_t k = 0; k < n; ++k) {
-    LBM_BCUDA(b, launch_lbm(b->prec == LBM_FP64, b->thermal, b->cols, MODE_STEP, b->launch_kernel, b->any_full,
+    LBM_BCUDA(b, launch_lbm(b->prec == LBM_FP64, b->thermal, b->cols, MODE_STEP, b->launch_kernel, b->flags,
                             b->d_insts, b->d_tiles, b->ntiles, b->stream, nullptr, b->max_polls));
     ++b->launches;
   }
@@ -217,7 +215,7 @@ lbm_status launch_steps(lbm_batch* b, int64_t n) {
 
 // CTAs one persistent launch of the batch may hold.
 long long batch_slots(const lbm_batch* b) {
-  return persistent_slots(b->prec == LBM_FP64, b->thermal, b->cols, b->launch_kernel, b->any_full, false);
+  return persistent_slots(b->prec == LBM_FP64, b->thermal, b->cols, b->launch_kernel, b->flags, false);
 }
 
 // Whether the batch's persistent launch overlaps consecutive steps (FlowPlan): every member
@@ -229,7 +227,7 @@ bool batch_overlapped(const lbm_batch* b) { return b->flow_ok && b->ntiles > bat
 // graph-replayed launches measured faster (served mixes of a few lattices: p50 time to result
 // 1.86 s against 1.97 s with a barrier between steps).
 bool batch_persistent(lbm_batch* b) {
-  if (b->launch_kernel != LBM_KERNEL_SCALAR && b->launch_kernel != LBM_KERNEL_INTERIOR) return false;
+  if (!has_persistent(b->launch_kernel)) return false;
   if (b->loop == LBM_LOOP_PERSISTENT) return true;
   if (b->loop == LBM_LOOP_LAUNCHES) return false;
   return b->flow_ok && 2 * (long long)b->ntiles >= 5 * batch_slots(b);
@@ -254,7 +252,7 @@ lbm_status launch_persistent_steps(lbm_batch* b, int64_t nsteps) {
       flow.cell_done = b->d_cells;
       LBM_BCUDA(b, cudaMemsetAsync(b->d_cells, 0, (size_t)b->ntiles * sizeof(unsigned long long), b->stream));
     }
-    LBM_BCUDA(b, launch_persistent(b->prec == LBM_FP64, b->thermal, b->cols, b->launch_kernel, b->any_full, b->d_insts,
+    LBM_BCUDA(b, launch_persistent(b->prec == LBM_FP64, b->thermal, b->cols, b->launch_kernel, b->flags, b->d_insts,
                                    b->d_tiles, b->ntiles, n, b->d_bar, b->max_polls, b->stream, nullptr, flow));
     ++b->launches;
     done += n;
@@ -267,7 +265,7 @@ lbm_status capture_graph(lbm_batch* b) {
   LBM_BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   lbm_status s = LBM_OK;
   for (int k = 0; k < kGraphChunk && s == LBM_OK; ++k) {
-    if (launch_lbm(b->prec == LBM_FP64, b->thermal, b->cols, MODE_STEP, b->launch_kernel, b->any_full, b->d_insts,
+    if (launch_lbm(b->prec == LBM_FP64, b->thermal, b->cols, MODE_STEP, b->launch_kernel, b->flags, b->d_insts,
                    b->d_tiles, b->ntiles, b->stream, nullptr, b->max_polls) != cudaSuccess)
       s = bfail(b, LBM_ECUDA, "launch during graph capture");
   }

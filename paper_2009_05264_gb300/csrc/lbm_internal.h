@@ -51,6 +51,64 @@ struct InstState {
                            // open ends (created minus lost populations), in slot n % 4
 };
 
+// D2Q9 weights.  In FP32 the rounded 4/9, 1/9, 1/36 sum to 1 + 7.6e-9, which would
+// create mass (and energy) in every collision in proportion to the stored deviation;
+// the FP32 set below (1/36 lowered by one ulp) sums to exactly 1.
+template <typename Real>
+struct LatWeights {
+  __host__ __device__ static constexpr Real w0() { return Real(4.0 / 9.0); }
+  __host__ __device__ static constexpr Real w1() { return Real(1.0 / 9.0); }
+  __host__ __device__ static constexpr Real w5() { return Real(1.0 / 36.0); }
+};
+template <>
+struct LatWeights<float> {
+  __host__ __device__ static constexpr float w0() { return 0x1.c71c72p-2f; }
+  __host__ __device__ static constexpr float w1() { return 0x1.c71c72p-4f; }
+  __host__ __device__ static constexpr float w5() { return 0x1.c71c70p-6f; }
+};
+// ---------------------------------------------------------------------------
+// Per-instance constants of the update, converted once per CTA to the compute
+// precision (the instance descriptor holds them in FP64).
+// ---------------------------------------------------------------------------
+template <typename Real>
+struct KConst {
+  Real omega_f, omega_g, a, b, R, kappa, inv_sqrtTc, psi_scale, beta, G2, Gh, mix, g_a, inv_cv;
+  Real T0, rho_ref, T_ref, alpha0, u_in, drho_out, dT_in, dT_heat;
+  // FP32 pseudopotential reference state (zero in FP64)
+  Real inv_u1r, inv_Dr, sqrtT_r, sa_r, rr2_Dr, rad_ref, psi_ref, p_ref;
+  // force on a row next to the bottom wall: wall0 + d * wall1 (the top wall: minus that)
+  Real wall0, wall1;
+  Real rho_ref_minus_avg;  // rho_ref - rho_avg of the previous step (buoyancy, Eq. 14)
+  Real drho_vapor;         // rho_vapor - rho_ref: vapour when drho < drho_vapor
+  // products of the constants above, formed once (host doubles): R / (1 - b rho_ref),
+  // a / D(rho_ref), 2 b rho_ref, -kappa / sqrt(Tc), a rho_ref^2 / D(rho_ref)
+  Real R_u1r, a_Dr, twob_rr, nk_sTc, a_rr2_Dr;
+};
+
+// Constants of the packed step, each held twice so that a packed instruction takes it as one
+// 64-bit operand; products are formed on the host in FP64.
+struct KPair {
+  float2 rho_ref, T_ref;
+  float2 b;  // Eq. 12
+  // with s = sqrt(alpha / alpha(T_ref)) = 1 + m1 (sqrt T - sqrt T_ref), D = 1 + 2 b rho - (b rho)^2:
+  // psi^2 - psi_ref^2 = cA (drho T / (1 - b rho) + rho_ref dT) + cB s^2 drho (s3 rho + rho_ref) / D
+  //                     + cK (s - 1) / m1 (s + 1) + c3 drho   (Eqs. 11, 12)
+  float2 m1, cA, cB, cK, c3, s3, T0;
+  float2 sqrtT_r, rad_ref, psi_ref;
+  float2 cR, cS;            // T (dp/dT)_rho / (rho c_v) = T (cR / (1 - b rho) + cS s / sqrt T rho / D)
+  float2 G2, Gh, Ghh;       // 2 G, G / 2, G / 4
+  float2 nbeta, npsi_ref, nmix;  // Eq. 8: -beta, -psi_ref, -(1 - beta) / 2
+  float2 ng_a, wall0, wall1;
+  float2 omega_f, keep_f, omega_g, keep_g;
+  float inv_ps, p_ref;              // probes only: dp = drad / psi_scale + drho / 3
+};
+
+// The converted constants of the FP32 strip step.
+struct StripConst {
+  KConst<float> C;
+  KPair P;
+};
+
 // Read-only description of one lattice instance (host-filled, device-resident).
 struct Inst {
   int nx, ny, pitch, geometry;
@@ -97,7 +155,91 @@ struct Inst {
   // a / D(rho_ref) with D(rho) = 1 + 2 b rho - (b rho)^2, 2 b rho_ref, -kappa / sqrt(Tc),
   // a rho_ref^2 / D(rho_ref)
   double R_u1r, a_Dr, twob_rr, nk_sTc, a_rr2_Dr;
+  StripConst strip;  // FP32; last: the one-column kernels copy what comes before it
 };
+
+// Every member is a conversion of a descriptor value (derived values are formed once, on the
+// host, in fill_inst), so the host's copy (kernel parameter) and a CTA's copy (shared memory)
+// are bit-identical.
+template <typename Real>
+__host__ __device__ inline void fill_consts(KConst<Real>& c, const Inst& I, double rho_avg_prev) {
+  c.omega_f = Real(I.omega_f);
+  c.omega_g = Real(I.omega_g);
+  c.a = Real(I.a);
+  c.b = Real(I.b);
+  c.R = Real(I.R);
+  c.kappa = Real(I.kappa);
+  c.inv_sqrtTc = Real(I.inv_sqrtTc);
+  c.psi_scale = Real(I.psi_scale);
+  c.beta = Real(I.beta);
+  c.G2 = Real(I.G2);
+  c.Gh = Real(I.Ghalf);
+  c.mix = Real(I.mix);
+  c.g_a = Real(I.g_a);
+  c.inv_cv = Real(I.inv_cv);
+  c.T0 = Real(I.T0);
+  c.rho_ref = Real(I.rho_ref);
+  c.T_ref = Real(I.T_ref);
+  c.alpha0 = Real(I.alpha0);
+  c.u_in = Real(I.u_in);
+  c.drho_out = Real(I.drho_out);
+  c.dT_in = Real(I.dT_in);
+  c.dT_heat = Real(I.dT_heat);
+  c.inv_u1r = Real(I.inv_u1r);
+  c.inv_Dr = Real(I.inv_Dr);
+  c.sqrtT_r = Real(I.sqrtT_r);
+  c.sa_r = Real(I.sa_r);
+  c.rr2_Dr = Real(I.rr2_Dr);
+  c.rad_ref = Real(I.rad_ref);
+  c.psi_ref = Real(I.psi_ref);
+  c.p_ref = Real(I.p_ref);
+  c.wall0 = Real(I.wall0);
+  c.wall1 = Real(I.wall1);
+  c.rho_ref_minus_avg = Real(I.rho_ref - rho_avg_prev);
+  c.drho_vapor = Real(I.drho_vapor);
+  c.R_u1r = Real(I.R_u1r);
+  c.a_Dr = Real(I.a_Dr);
+  c.twob_rr = Real(I.twob_rr);
+  c.nk_sTc = Real(I.nk_sTc);
+  c.a_rr2_Dr = Real(I.a_rr2_Dr);
+}
+
+__host__ __device__ inline float2 pair_of(double v) { return make_float2((float)v, (float)v); }
+
+__host__ __device__ inline void fill_pair_consts(KPair& P, const Inst& I) {
+  const double ps = I.psi_scale, sr = I.sa_r;
+  P.rho_ref = pair_of(I.rho_ref);
+  P.T_ref = pair_of(I.T_ref);
+  P.b = pair_of(I.b);
+  P.m1 = pair_of(sr != 0.0 ? I.nk_sTc / sr : 0.0);
+  P.cA = pair_of(I.R_u1r * ps);
+  P.cB = pair_of(-I.a_Dr * sr * sr * ps);
+  P.cK = pair_of(-I.a_rr2_Dr * I.nk_sTc * sr * ps);
+  P.c3 = pair_of(-ps / 3.0);
+  P.s3 = pair_of(1.0 + I.twob_rr);
+  P.T0 = pair_of(I.T0);
+  P.sqrtT_r = pair_of(I.sqrtT_r);
+  P.rad_ref = pair_of(I.rad_ref);
+  P.psi_ref = pair_of(I.psi_ref);
+  P.cR = pair_of(I.R * I.inv_cv);
+  P.cS = pair_of(-I.a * I.nk_sTc * sr * I.inv_cv);
+  P.G2 = pair_of(I.G2);
+  P.Gh = pair_of(I.Ghalf);
+  P.Ghh = pair_of(0.5 * I.Ghalf);
+  P.nbeta = pair_of(-I.beta);
+  P.npsi_ref = pair_of(-I.psi_ref);
+  P.nmix = pair_of(-I.mix);
+  P.ng_a = pair_of(-I.g_a);
+  P.wall0 = pair_of(I.wall0);
+  P.wall1 = pair_of(I.wall1);
+  P.omega_f = pair_of(I.omega_f);
+  // 1 - omega of the FP32 omega, exactly: a collision must not create mass or energy
+  P.keep_f = make_float2(1.0f - P.omega_f.x, 1.0f - P.omega_f.x);
+  P.omega_g = pair_of(I.omega_g);
+  P.keep_g = make_float2(1.0f - P.omega_g.x, 1.0f - P.omega_g.x);
+  P.inv_ps = ps != 0.0 ? (float)(1.0 / ps) : 0.0f;
+  P.p_ref = (float)I.p_ref;
+}
 
 // State of the grid-wide barrier between the steps of a persistent launch (device memory,
 // zeroed by the host before every persistent launch).  count: CTAs arrived at the current
@@ -157,43 +299,60 @@ inline int tile_is_interior(int geometry, int nx, int cols, int x0) {
 inline bool general_tile(const Tile& t) { return !t.interior; }
 
 // Launchers (defined per precision).  Tiles must have been built for `cols`.
-// kernel: a resolved form (resolve_kernel): LBM_KERNEL_SCALAR, _INTERIOR, _PAIRED or _TMA.
-// full: the instances use the pool geometry, the Hazi-Markus source or bubble statistics, which
-// only the step's full form handles (the lean form leaves them out of the hot loop).
+// kernel: a resolved form (resolve_kernel): LBM_KERNEL_SCALAR, _INTERIOR, _TMA or FORM_STRIP.
+// flags: STEP_FULL, the instances use the pool geometry, the Hazi-Markus source or bubble
+// statistics, which only the step's full form handles (the lean form leaves them out of the hot
+// loop); STEP_RELAX, tau_f != 1 (the strip kernel then keeps the pulled f for the collision).
 // h_inst: host copy of the launch's only instance (the lean scalar step then takes its
 // constants as a kernel parameter), or null for launches over several instances.
 // max_polls: poll cap of the TMA form's row waits (0: its full limit; lbm_set_wait_limit).
-cudaError_t launch_lbm(int fp64, int thermal, int cols, int mode, int kernel, bool full, const Inst* d_inst,
+cudaError_t launch_lbm(int fp64, int thermal, int cols, int mode, int kernel, int flags, const Inst* d_inst,
                        const Tile* d_tiles, int ntiles, cudaStream_t s, const Inst* h_inst = nullptr,
                        unsigned max_polls = 0);
 // nsteps steps of the step kernel in one cooperative launch (tiles drawn dynamically from a
 // counter, a bounded grid barrier between steps; MODE_STEP only).  grid <= resident CTAs of
 // the device; bar: zeroed GridBar in device memory.
 // flow.enabled: the overlapped form (one instance; more tiles than resident CTAs).
-cudaError_t launch_persistent(int fp64, int thermal, int cols, int kernel, bool full, const Inst* d_inst,
+cudaError_t launch_persistent(int fp64, int thermal, int cols, int kernel, int flags, const Inst* d_inst,
                               const Tile* d_tiles, int ntiles, int nsteps, GridBar* bar, unsigned max_polls,
                               cudaStream_t s, const Inst* h_inst, const FlowPlan& flow);
 // CTAs one persistent launch may hold on the current device (SMs x resident CTAs per SM).
-long long persistent_slots(int fp64, int thermal, int cols, int kernel, bool full, bool single);
+long long persistent_slots(int fp64, int thermal, int cols, int kernel, int flags, bool single);
 // Whether an instance needs the step's full form.
 inline bool needs_full_step(const Inst& I) {
   return I.geometry == GEOM_POOL || I.source_model != 0 || I.bubble_stats != 0;
 }
-// The step-kernel form a launch takes for a requested LBM_KERNEL_* value.  LBM_KERNEL_AUTO
-// and LBM_KERNEL_INTERIOR take the one-column kernel with its interior path (tiles away from
-// open ends and wraps run a loop without any per-node boundary logic; the others run the
-// general loop), the fastest form on GB300, whenever the step's lean form applies, else the
-// plain one-column kernel.  FP64 has no other forms; the paired kernel has no Hazi-Markus
-// source; the TMA kernel needs 128-column tiles, the step's lean form and the instances'
-// tensor maps (tmaps: all instances of the launch have them).
+enum : int { STEP_FULL = 1, STEP_RELAX = 2 };
+inline int step_flags(const Inst& I) {
+  return (needs_full_step(I) ? STEP_FULL : 0) | (I.omega_f != 1.0 ? STEP_RELAX : 0);
+}
+// The kernel a launch takes for a requested LBM_KERNEL_* value.  In FP32, LBM_KERNEL_AUTO,
+// _INTERIOR and _PAIRED all take the strip kernel (lbm_strip.cuh), which handles every option and
+// is the fastest on GB300.  In FP64, LBM_KERNEL_AUTO and _INTERIOR take the one-column kernel
+// with its interior path (tiles away from open ends and wraps run a loop without any per-node
+// boundary logic; the others run the general loop) whenever the step's lean form applies, else
+// the plain one-column kernel.  The TMA kernel needs FP32, 128-column tiles, the step's lean form
+// and the instances' tensor maps (tmaps: all instances of the launch have them).
 constexpr int TMA_TILE_COLS = 128;
-inline int resolve_kernel(int requested, int fp64, bool full, bool hazi, bool tmaps, int cols) {
+constexpr int FORM_STRIP = 16;  // beside the LBM_KERNEL_* values
+inline int resolve_kernel(int requested, int fp64, bool full, bool tmaps, int cols) {
   if (requested == LBM_KERNEL_AUTO || requested == LBM_KERNEL_INTERIOR)
-    return full ? LBM_KERNEL_SCALAR : LBM_KERNEL_INTERIOR;
+    return !fp64 ? FORM_STRIP : full ? LBM_KERNEL_SCALAR : LBM_KERNEL_INTERIOR;
   if (fp64) return LBM_KERNEL_SCALAR;
-  if (requested == LBM_KERNEL_PAIRED) return hazi ? LBM_KERNEL_SCALAR : LBM_KERNEL_PAIRED;
+  if (requested == LBM_KERNEL_PAIRED) return FORM_STRIP;
   if (requested == LBM_KERNEL_TMA && !full && tmaps && cols == TMA_TILE_COLS) return LBM_KERNEL_TMA;
   return LBM_KERNEL_SCALAR;
+}
+// The LBM_KERNEL_* value reported for it: the strip kernel goes by the form that was asked for,
+// "scalar" where that form's boundary logic is the per-node one (the full form, Hazi-Markus).
+inline int reported_kernel(int requested, int form, bool full, bool hazi) {
+  if (form != FORM_STRIP) return form;
+  if (requested == LBM_KERNEL_PAIRED) return hazi ? LBM_KERNEL_SCALAR : LBM_KERNEL_PAIRED;
+  return full ? LBM_KERNEL_SCALAR : LBM_KERNEL_INTERIOR;
+}
+// Whether a kernel has a persistent form.
+inline bool has_persistent(int form) {
+  return form == LBM_KERNEL_SCALAR || form == LBM_KERNEL_INTERIOR || form == FORM_STRIP;
 }
 // f = f^eq(rho,u), g = g^eq(T,u) into buffer 0 from 4 planes of nx*ny doubles (rho, ux, uy, T).
 cudaError_t launch_init_from_fields(int fp64, const Inst* d_inst, int nx, int ny, const double* d_fields,
@@ -235,8 +394,8 @@ struct BandPlan {
 BandPlan default_band_plan(int nx, int ny, int cols, long long slots);
 // CTAs of the step kernel (storage precision, thermal flag, tile columns, kernel
 // form) that one wave of the current device holds: SMs x resident CTAs per SM.
-long long step_wave_slots(int fp64, int thermal, int cols, int kernel);
-int resident_ctas_f32(int thermal, int cols, int kernel);
+long long step_wave_slots(int fp64, int thermal, int cols, int kernel, int flags = 0);
+int resident_ctas_f32(int thermal, int cols, int kernel, int flags);
 int resident_ctas_f64(int thermal, int cols, int kernel);
 // The instance descriptor of a context (device pointers included), for batching.
 Inst lbm_internal_inst(const lbm_ctx* c);

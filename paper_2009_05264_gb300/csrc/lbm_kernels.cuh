@@ -33,6 +33,7 @@
 
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "lbm_internal.h"
@@ -48,21 +49,6 @@ __host__ __device__ constexpr int lat_cy(int i) {
 __host__ __device__ constexpr int lat_opp(int i) {
   return i == 0 ? 0 : (i <= 4 ? ((i + 1) % 4) + 1 : ((i - 3) % 4) + 5);
 }
-// D2Q9 weights.  In FP32 the rounded 4/9, 1/9, 1/36 sum to 1 + 7.6e-9, which would
-// create mass (and energy) in every collision in proportion to the stored deviation;
-// the FP32 set below (1/36 lowered by one ulp) sums to exactly 1.
-template <typename Real>
-struct LatWeights {
-  __host__ __device__ static constexpr Real w0() { return Real(4.0 / 9.0); }
-  __host__ __device__ static constexpr Real w1() { return Real(1.0 / 9.0); }
-  __host__ __device__ static constexpr Real w5() { return Real(1.0 / 36.0); }
-};
-template <>
-struct LatWeights<float> {
-  __host__ __device__ static constexpr float w0() { return 0x1.c71c72p-2f; }
-  __host__ __device__ static constexpr float w1() { return 0x1.c71c72p-4f; }
-  __host__ __device__ static constexpr float w5() { return 0x1.c71c70p-6f; }
-};
 template <typename Real>
 __host__ __device__ constexpr Real lat_w(int i) {
   return i == 0 ? LatWeights<Real>::w0() : (i <= 4 ? LatWeights<Real>::w1() : LatWeights<Real>::w5());
@@ -73,8 +59,16 @@ __device__ __forceinline__ int wrap_index(int v, int n) {
   return v < 0 ? v + n : v;
 }
 
-__device__ __forceinline__ float ld_ro(const float* p) { return __ldg(p); }
-__device__ __forceinline__ double ld_ro(const double* p) { return __ldg(p); }
+// Loads of single populations in the boundary conditions, from L2: in a persistent launch other
+// CTAs write them during the launch.
+__device__ __forceinline__ float ld_ro(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ double ld_ro(const double* p) { return __ldcg(p); }
+
+// Pressure probe j of a step (visible before the tile's ticket).
+__device__ __forceinline__ void st_probe(InstState* st, int j, float p) {
+  st->p_probe[j] = (double)p;
+  __threadfence();
+}
 
 // Bounds-checked build (compiled with -DLBM_BOUNDS_CHECK, for tests): before each global access
 // of the step and initialisation kernels, idx_ok checks the element index k against the n
@@ -177,71 +171,6 @@ constexpr size_t step_smem_bytes() {
   return INTERIOR && interior_smem_bytes<Real, THERMAL, B>() > fused_smem_bytes<Real, THERMAL, B>()
              ? interior_smem_bytes<Real, THERMAL, B>()
              : fused_smem_bytes<Real, THERMAL, B>();
-}
-
-// ---------------------------------------------------------------------------
-// Per-instance constants of the update, converted once per CTA to the compute
-// precision (the instance descriptor holds them in FP64).
-// ---------------------------------------------------------------------------
-template <typename Real>
-struct KConst {
-  Real omega_f, omega_g, a, b, R, kappa, inv_sqrtTc, psi_scale, beta, G2, Gh, mix, g_a, inv_cv;
-  Real T0, rho_ref, T_ref, alpha0, u_in, drho_out, dT_in, dT_heat;
-  // FP32 pseudopotential reference state (zero in FP64)
-  Real inv_u1r, inv_Dr, sqrtT_r, sa_r, rr2_Dr, rad_ref, psi_ref, p_ref;
-  // force on a row next to the bottom wall: wall0 + d * wall1 (the top wall: minus that)
-  Real wall0, wall1;
-  Real rho_ref_minus_avg;  // rho_ref - rho_avg of the previous step (buoyancy, Eq. 14)
-  Real drho_vapor;         // rho_vapor - rho_ref: vapour when drho < drho_vapor
-  // products of the constants above, formed once (host doubles): R / (1 - b rho_ref),
-  // a / D(rho_ref), 2 b rho_ref, -kappa / sqrt(Tc), a rho_ref^2 / D(rho_ref)
-  Real R_u1r, a_Dr, twob_rr, nk_sTc, a_rr2_Dr;
-};
-
-// Every member is a conversion of a descriptor value (derived values are formed once, on the
-// host, in fill_inst), so the host's copy (kernel parameter) and a CTA's copy (shared memory)
-// are bit-identical.
-template <typename Real>
-__host__ __device__ inline void fill_consts(KConst<Real>& c, const Inst& I, double rho_avg_prev) {
-  c.omega_f = Real(I.omega_f);
-  c.omega_g = Real(I.omega_g);
-  c.a = Real(I.a);
-  c.b = Real(I.b);
-  c.R = Real(I.R);
-  c.kappa = Real(I.kappa);
-  c.inv_sqrtTc = Real(I.inv_sqrtTc);
-  c.psi_scale = Real(I.psi_scale);
-  c.beta = Real(I.beta);
-  c.G2 = Real(I.G2);
-  c.Gh = Real(I.Ghalf);
-  c.mix = Real(I.mix);
-  c.g_a = Real(I.g_a);
-  c.inv_cv = Real(I.inv_cv);
-  c.T0 = Real(I.T0);
-  c.rho_ref = Real(I.rho_ref);
-  c.T_ref = Real(I.T_ref);
-  c.alpha0 = Real(I.alpha0);
-  c.u_in = Real(I.u_in);
-  c.drho_out = Real(I.drho_out);
-  c.dT_in = Real(I.dT_in);
-  c.dT_heat = Real(I.dT_heat);
-  c.inv_u1r = Real(I.inv_u1r);
-  c.inv_Dr = Real(I.inv_Dr);
-  c.sqrtT_r = Real(I.sqrtT_r);
-  c.sa_r = Real(I.sa_r);
-  c.rr2_Dr = Real(I.rr2_Dr);
-  c.rad_ref = Real(I.rad_ref);
-  c.psi_ref = Real(I.psi_ref);
-  c.p_ref = Real(I.p_ref);
-  c.wall0 = Real(I.wall0);
-  c.wall1 = Real(I.wall1);
-  c.rho_ref_minus_avg = Real(I.rho_ref - rho_avg_prev);
-  c.drho_vapor = Real(I.drho_vapor);
-  c.R_u1r = Real(I.R_u1r);
-  c.a_Dr = Real(I.a_Dr);
-  c.twob_rr = Real(I.twob_rr);
-  c.nk_sTc = Real(I.nk_sTc);
-  c.a_rr2_Dr = Real(I.a_rr2_Dr);
 }
 
 // Kernel parameter of a launch over one instance: its descriptor and converted constants.
@@ -389,28 +318,15 @@ struct NodeState {
 // (dp/dT)_rho of one node.  In FP32 psi is evaluated as psi - psi_ref from exact
 // difference forms of Eq. 12 in rho - rho_ref and T - T_ref, so that neighbour
 // differences in the force keep their low-order bits.
-// PAIRED (FP32 thermal, interior path): the two sums of Eqs. 4 and 17 in the two lanes of
-// paired FP32 additions (same association, each lane rounded as before).
-template <typename Real, bool THERMAL, bool PAIRED = false>
+template <typename Real, bool THERMAL>
 __device__ __forceinline__ NodeState<Real> node_state(const Real (&fc)[9], const Real (&gc)[9],
                                                       const KConst<Real>& C, bool multiphase, bool hazi = false) {
   NodeState<Real> o;
   o.hmc = Real(0);
   const Real rho_ref = C.rho_ref;
   Real sum_g = Real(0);
-  if constexpr (PAIRED && THERMAL && sizeof(Real) == 4) {
-    float2 q[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) q[i] = make_float2(fc[i], gc[i]);
-    const float2 sum = __fadd2_rn(__fadd2_rn(__fadd2_rn(__fadd2_rn(q[0], q[1]), __fadd2_rn(q[2], q[3])),
-                                             __fadd2_rn(__fadd2_rn(q[4], q[5]), __fadd2_rn(q[6], q[7]))),
-                                  q[8]);
-    o.drho = sum.x;
-    sum_g = sum.y;
-  } else {
-    o.drho = ((fc[0] + fc[1]) + (fc[2] + fc[3])) + ((fc[4] + fc[5]) + (fc[6] + fc[7])) + fc[8];
-    if (THERMAL) sum_g = ((gc[0] + gc[1]) + (gc[2] + gc[3])) + ((gc[4] + gc[5]) + (gc[6] + gc[7])) + gc[8];
-  }
+  o.drho = ((fc[0] + fc[1]) + (fc[2] + fc[3])) + ((fc[4] + fc[5]) + (fc[6] + fc[7])) + fc[8];
+  if (THERMAL) sum_g = ((gc[0] + gc[1]) + (gc[2] + gc[3])) + ((gc[4] + gc[5]) + (gc[6] + gc[7])) + gc[8];
   o.rho = rho_ref + o.drho;
   const Real jx = (fc[1] - fc[3]) + (fc[5] - fc[6]) + (fc[8] - fc[7]);
   const Real jy = (fc[2] - fc[4]) + (fc[5] + fc[6]) - (fc[7] + fc[8]);
@@ -504,33 +420,6 @@ __device__ __forceinline__ void sc_force(Real dc, Real dE, Real dW, Real dN, Rea
   const Real lead = C.psi_ref + C.beta * dc;
   Fx = -lead * t1x - C.mix * t2x;
   Fy = -lead * t1y - C.mix * t2y;
-  if (sol_m) Fy += C.wall0 + dc * C.wall1;
-  if (sol_p) Fy -= C.wall0 + dc * C.wall1;
-}
-
-// FP32 form of sc_force for the interior path, with paired FP32 instructions: the x and y
-// components in the two lanes of a register pair, and the diagonal neighbours' sums and
-// differences formed two at a time.  The same expressions as sc_force (the products keep its
-// difference-of-squares form (a - b)(a + b)); only the grouping of the roundings differs.
-__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
-
-__device__ __forceinline__ void sc_force_paired(float dc, float dE, float dW, float dN, float dNE, float dNW, float dS,
-                                                float dSE, float dSW, bool sol_m, bool sol_p, const KConst<float>& C,
-                                                float& Fx, float& Fy) {
-  const float2 P = make_float2(dE, dN), Q = make_float2(dW, dS);
-  const float2 A = f2sub(P, Q), S = __fadd2_rn(P, Q);        // (dE - dW, dN - dS), (dE + dW, dN + dS)
-  const float2 U = make_float2(dNE, dSE), V = make_float2(dNW, dSW);
-  const float2 m = f2sub(U, V), p = __fadd2_rn(U, V);        // (dNE - dNW, dSE - dSW), (dNE + dNW, dSE + dSW)
-  const float2 U2 = make_float2(dNE, dNW), V2 = make_float2(dSE, dSW);
-  const float2 b = f2sub(U2, V2), a = __fadd2_rn(U2, V2);    // (dNE - dSE, dNW - dSW), (dNE + dSE, dNW + dSW)
-  const float2 mp = __fmul2_rn(m, p), ab = __fmul2_rn(b, a);
-  const float2 G2 = make_float2(C.G2, C.G2), Gh = make_float2(C.Gh, C.Gh);
-  const float2 t1 = __ffma2_rn(G2, A, __fmul2_rn(Gh, make_float2(m.x + m.y, p.x - p.y)));
-  const float2 t2 = __ffma2_rn(__fmul2_rn(G2, A), S, __fmul2_rn(Gh, make_float2(mp.x + mp.y, ab.x + ab.y)));
-  const float nlead = -(C.psi_ref + C.beta * dc);
-  const float2 F = __ffma2_rn(make_float2(nlead, nlead), t1, __fmul2_rn(make_float2(-C.mix, -C.mix), t2));
-  Fx = F.x;
-  Fy = F.y;
   if (sol_m) Fy += C.wall0 + dc * C.wall1;
   if (sol_p) Fy -= C.wall0 + dc * C.wall1;
 }
@@ -637,73 +526,6 @@ __device__ __forceinline__ void collide_g(const Pops& gs, const Out& go, Real T,
   pair(2, 4, uay, lat_w<Real>(2));
   pair(5, 7, uax + uay, lat_w<Real>(5));
   pair(6, 8, uay - uax, lat_w<Real>(6));
-}
-
-// FP32 forms of the two collisions for the interior path, with paired FP32 arithmetic
-// (FADD2 / FMUL2 / FFMA2: two independent operations per instruction).  The pairs of
-// opposite directions that share a weight are computed two at a time: the axis pairs
-// (1,3) and (2,4) in the two lanes of one register pair, the diagonal pairs (5,7) and (6,8)
-// in another.  Same formulas as collide_f / collide_g; only the grouping of the roundings
-// differs (paired instructions round each lane exactly as the scalar instruction would).
-__device__ __forceinline__ float2 f2bc(float a) { return make_float2(a, a); }
-
-template <typename Pops, typename Out>
-__device__ __forceinline__ void collide_f_paired(const Pops& fs, const Out& fo, float rho, float drho, float ux,
-                                                 float uy, float dux, float duy, float omega_f) {
-  constexpr float w0 = LatWeights<float>::w0(), w1 = LatWeights<float>::w1(), w5 = LatWeights<float>::w5();
-  const float2 U = make_float2(ux, uy), D = make_float2(dux, duy);
-  const float2 S = __ffma2_rn(f2bc(2.0f), U, D);  // (2u + du) per axis
-  const float2 UU = __fmul2_rn(U, U);
-  const float2 DS = __fmul2_rn(D, S);
-  const float r15 = 1.5f * rho;
-  const float K = omega_f * (drho - r15 * (UU.x + UU.y)) - r15 * (DS.x + DS.y);
-  const float r45 = 4.5f * rho, r3 = 3.0f * rho, keep = 1.0f - omega_f;
-  fo(0) = keep * fs(0) + w0 * K;
-  const float2 KEEP = f2bc(keep), R45 = f2bc(r45), KK = f2bc(K), WF = f2bc(omega_f), NEG = f2bc(-1.0f);
-  auto pairs = [&](float2 cu, float2 cd, float2 cs, float w, int i, int j, int ib, int jb) {
-    const float2 wcu = __fmul2_rn(WF, cu);                                     // omega c.u
-    const float2 X = __ffma2_rn(wcu, cu, __fmul2_rn(cd, cs));                  // omega cu^2 + cd cs
-    const float2 sym = __fmul2_rn(f2bc(w), __ffma2_rn(R45, X, KK));           // w (K + 4.5 rho X)
-    const float2 anti = __fmul2_rn(f2bc(w * r3), __fadd2_rn(wcu, cd));        // 3 w rho (omega cu + cd)
-    const float2 plus = __fadd2_rn(sym, anti), minus = __ffma2_rn(anti, NEG, sym);
-    const float2 a = __ffma2_rn(KEEP, make_float2(fs(i), fs(j)), plus);
-    const float2 b = __ffma2_rn(KEEP, make_float2(fs(ib), fs(jb)), minus);
-    fo(i) = a.x;
-    fo(j) = a.y;
-    fo(ib) = b.x;
-    fo(jb) = b.y;
-  };
-  pairs(U, D, S, w1, 1, 2, 3, 4);  // lanes: (1,3) with c.u = ux, (2,4) with c.u = uy
-  const float2 PM = make_float2(1.0f, -1.0f);
-  const float2 Ud = __ffma2_rn(f2bc(ux), PM, f2bc(uy));    // (ux + uy, uy - ux)
-  const float2 Dd = __ffma2_rn(f2bc(dux), PM, f2bc(duy));
-  const float2 Sd = __ffma2_rn(f2bc(S.x), PM, f2bc(S.y));
-  pairs(Ud, Dd, Sd, w5, 5, 6, 7, 8);  // lanes: (5,7) with c.u = ux + uy, (6,8) with c.u = uy - ux
-}
-
-template <typename Pops, typename Out>
-__device__ __forceinline__ void collide_g_paired(const Pops& gs, const Out& go, float T, float dT, float uax,
-                                                 float uay, float phi, float omega_g) {
-  constexpr float w0 = LatWeights<float>::w0(), w1 = LatWeights<float>::w1(), w5 = LatWeights<float>::w5();
-  const float2 U = make_float2(uax, uay);
-  const float2 UU = __fmul2_rn(U, U);
-  const float Kg = omega_g * (dT - 1.5f * T * (UU.x + UU.y)) + phi;
-  const float t45 = 4.5f * omega_g * T, t3 = 3.0f * omega_g * T, keep = 1.0f - omega_g;
-  go(0) = keep * gs(0) + w0 * Kg;
-  const float2 KEEP = f2bc(keep), NEG = f2bc(-1.0f);
-  auto pairs = [&](float2 cu, float w, int i, int j, int ib, int jb) {
-    const float2 sym = __ffma2_rn(f2bc(w * t45), __fmul2_rn(cu, cu), f2bc(w * Kg));  // w (Kg + 4.5 omega T cu^2)
-    const float2 anti = __fmul2_rn(f2bc(w * t3), cu);                                 // 3 w omega T cu
-    const float2 plus = __fadd2_rn(sym, anti), minus = __ffma2_rn(anti, NEG, sym);
-    const float2 a = __ffma2_rn(KEEP, make_float2(gs(i), gs(j)), plus);
-    const float2 b = __ffma2_rn(KEEP, make_float2(gs(ib), gs(jb)), minus);
-    go(i) = a.x;
-    go(j) = a.y;
-    go(ib) = b.x;
-    go(jb) = b.y;
-  };
-  pairs(U, w1, 1, 2, 3, 4);
-  pairs(__ffma2_rn(f2bc(uax), make_float2(1.0f, -1.0f), f2bc(uay)), w5, 5, 6, 7, 8);
 }
 
 // Issue the asynchronous pull of one node's populations into f_dst/g_dst (stride
@@ -830,11 +652,12 @@ __device__ __forceinline__ void finish_step(const Inst& I, InstState* st, const 
 // step's buoyancy mean from it); the fixed-point grid is the inflow total's.  NA: the partials
 // the tile can have nonzero (the first NA of acc; an interior tile has mass, energy and the
 // heater row only); a total that a tile leaves at zero takes no atomic.
-template <int BLOCK, bool THERMAL, int MODE, int NA = NPART>
+// WARPS: the most warps a CTA of the kernel has.
+template <int WARPS, bool THERMAL, int MODE, int NA = NPART>
 __device__ __forceinline__ void post_partials(const Inst& I, InstState* st, const Tile& tile, const double (&acc)[NPART],
                                               double (*red)[NPART], int* flag, long long step, bool open = false,
                                               double open_acc = 0.0) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   unsigned long long* const sums = I.sums + (step & 1) * NPART;
 #pragma unroll
   for (int j = 0; j < NA; ++j) {
@@ -847,12 +670,12 @@ __device__ __forceinline__ void post_partials(const Inst& I, InstState* st, cons
     double x = open_acc;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    __shared__ double s_open[BLOCK / 32];
+    __shared__ double s_open[WARPS];
     if (lane == 0) s_open[warp] = x;
     __syncthreads();
     if (tid == 0) {
       double sum = 0.0;
-      for (int w = 0; w < BLOCK / 32; ++w) sum += s_open[w];
+      for (int w = 0; w < nwarps; ++w) sum += s_open[w];
       const double q = sum * I.fix_scale[3];
       long long v = 0;
       if (fabs(q) < 0x1p62) v = __double2ll_rn(q);
@@ -865,7 +688,7 @@ __device__ __forceinline__ void post_partials(const Inst& I, InstState* st, cons
   __syncthreads();
   if (tid < NA) {
     double sum = 0.0;
-    for (int w = 0; w < BLOCK / 32; ++w) sum += red[w][tid];
+    for (int w = 0; w < nwarps; ++w) sum += red[w][tid];
     const double x = sum * I.fix_scale[tid];  // a power of two: exact
     long long q = 0;
     if (fabs(x) < 0x1p62) q = __double2ll_rn(x);
@@ -1030,7 +853,7 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
 #pragma unroll
         for (int i = 0; i < 9; ++i) gs[i * NS] = gc[i];
       }
-      ns = node_state<Real, THERMAL, true>(fc, gc, C, multiphase, false);
+      ns = node_state<Real, THERMAL>(fc, gc, C, multiphase, false);
       bad_any = bad_any || ns.bad;
       sPsi[p_cur * NS + s] = ns.dpsi;
       if (out_col && r >= y0 && r < y1) {
@@ -1052,10 +875,7 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
         const Real* Pp = sPsi + p_cur * NS + s;
         const Real* Pm = sPsi + p_prev2 * NS + s;
         auto force = [&](Real dN, Real dNE, Real dNW, Real dS, Real dSE, Real dSW, bool sol_m, bool sol_p) {
-          if constexpr (sizeof(Real) == 4)
-            sc_force_paired(P0[0], P0[1], P0[-1], dN, dNE, dNW, dS, dSE, dSW, sol_m, sol_p, C, Fx, Fy);
-          else
-            sc_force<Real>(P0[0], P0[1], P0[-1], dN, dNE, dNW, dS, dSE, dSW, sol_m, sol_p, C, Fx, Fy);
+          sc_force<Real>(P0[0], P0[1], P0[-1], dN, dNE, dNW, dS, dSE, dSW, sol_m, sol_p, C, Fx, Fy);
         };
         if (q > 0 && q < ny - 1) {
           force(Pp[0], Pp[1], Pp[-1], Pm[0], Pm[1], Pm[-1], false, false);
@@ -1072,11 +892,7 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
       sUx[p_prev * NS + s] = uax;
       sUy[p_prev * NS + s] = uay;
       if (out_col && q >= y0 && q < y1) {
-        if constexpr (sizeof(Real) == 4)
-          collide_f_paired(StridedPops<Real>{sF + f_prev * 9 * NS + s, NS}, OffsetOut<Real>{Fout, q * pitch + xn, I},
-                           rho_p, drho_p, ux_p, uy_p, dux, duy, C.omega_f);
-        else
-          collide_f<Real>(StridedPops<Real>{sF + f_prev * 9 * NS + s, NS}, OffsetOut<Real>{Fout, q * pitch + xn, I},
+        collide_f<Real>(StridedPops<Real>{sF + f_prev * 9 * NS + s, NS}, OffsetOut<Real>{Fout, q * pitch + xn, I},
                           rho_p, drho_p, ux_p, uy_p, dux, duy, C.omega_f);
       }
     }
@@ -1099,11 +915,7 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
         }
         const Real divu = Real(0.5) * (uxE - uxW) + dyu;
         const Real phi = coef_p2 * divu;
-        if constexpr (sizeof(Real) == 4)
-          collide_g_paired(StridedPops<Real>{sG + g_prev2 * 9 * NS + s, NS}, OffsetOut<Real>{Gout, q2 * pitch + xn, I},
-                           T_p2, dT_p2, U2x[0], U2y[0], phi, C.omega_g);
-        else
-          collide_g<Real>(StridedPops<Real>{sG + g_prev2 * 9 * NS + s, NS}, OffsetOut<Real>{Gout, q2 * pitch + xn, I},
+        collide_g<Real>(StridedPops<Real>{sG + g_prev2 * 9 * NS + s, NS}, OffsetOut<Real>{Gout, q2 * pitch + xn, I},
                           T_p2, dT_p2, U2x[0], U2y[0], phi, C.omega_g);
       }
     }
@@ -1206,7 +1018,7 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
   if constexpr (!PCONST) {
     const int* src = reinterpret_cast<const int*>(insts + tile.inst);
     int* dst = reinterpret_cast<int*>(&sh.sI);
-    for (int k = tid; k < (int)(sizeof(Inst) / 4); k += BLOCK) dst[k] = src[k];
+    for (int k = tid; k < (int)(offsetof(Inst, strip) / 4); k += BLOCK) dst[k] = src[k];
     __syncthreads();
   }
   const Inst& I = tile_inst<Real, B, PCONST>(kp, sh);
@@ -1230,7 +1042,7 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
     interior_rows<Real, THERMAL, B>(I, sC, sRra, tile, step, local, dyn_smem, am, ae, ah, bad_any);
     if (bad_any) atomicOr(&st->status, STATUS_UNSTABLE);
     const double acc[NPART] = {(double)am, (double)ae, (double)ah, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    post_partials<BLOCK, THERMAL, MODE, 3>(I, st, tile, acc, sRed, &sLast, step);
+    post_partials<BLOCK / 32, THERMAL, MODE, 3>(I, st, tile, acc, sRed, &sLast, step);
     return;
   }
   const bool perx = I.geometry != GEOM_CHANNEL;
@@ -1495,20 +1307,17 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
   // ---------------- per-tile partials into the launch's totals ----------------
   double acc[NPART] = {(double)acc_m,  (double)acc_e,  (double)acc_h,  (double)acc_fi, (double)acc_fo,
                        (double)acc_va, (double)acc_wv, (double)acc_hv, (double)acc_zv};
-  post_partials<BLOCK, THERMAL, MODE>(I, st, tile, acc, sRed, &sLast, step, post_open, acc_open);
+  post_partials<BLOCK / 32, THERMAL, MODE>(I, st, tile, acc, sRed, &sLast, step, post_open, acc_open);
 }
 
-// Resident CTAs per SM the step kernels are compiled for (register budget).  The FP32 kernel
-// with the interior path is compiled for 4 CTAs of 128 threads per SM (up to 128 registers):
-// measured faster than 5 at 96 registers or 6 at 80, both of which also leave less L1 beside
-// the shared-memory rings.
-template <typename Real, int B, bool INTERIOR>
+// Resident CTAs per SM the step kernels are compiled for (register budget).
+template <typename Real, int B>
 constexpr int step_min_blocks() {
-  return sizeof(Real) == 4 ? (B <= 64 ? 10 : (B <= 128 ? (INTERIOR ? 4 : 5) : 2)) : (B <= 64 ? 4 : (B <= 128 ? 2 : 1));
+  return sizeof(Real) == 4 ? (B <= 64 ? 10 : (B <= 128 ? 5 : 2)) : (B <= 64 ? 4 : (B <= 128 ? 2 : 1));
 }
 
 template <typename Real, bool THERMAL, int B, int MODE, bool FULL = true, bool PCONST = false, bool INTERIOR = false>
-__global__ void __launch_bounds__(B, (step_min_blocks<Real, B, INTERIOR>()))
+__global__ void __launch_bounds__(B, (step_min_blocks<Real, B>()))
 lbm_fused_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles,
                  const __grid_constant__ KParams<Real> kp) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -1600,19 +1409,20 @@ __device__ __forceinline__ bool flow_wait(const volatile T* p, T need, const Gri
 // Tickets are drawn in order and a tile waits only for tickets drawn before it, all of them
 // held by resident CTAs, so the loop always progresses; a CTA that gives up marks the launch
 // (bar->status), every CTA then stops at its next wait, and the instance reports a timeout.
-template <typename Real, bool THERMAL, int B, bool FULL, bool PCONST, bool INTERIOR>
-__device__ __forceinline__ void overlapped_steps(const Inst* __restrict__ insts, const Tile* __restrict__ tiles,
-                                                 int ntiles, int nsteps, GridBar* bar, unsigned max_polls,
-                                                 const KParams<Real>& kp, const FlowPlan& flow,
-                                                 unsigned char* dyn_smem, StepShared<Real, B, PCONST>& sh) {
+// single: the launch's only instance (its descriptor as a kernel parameter), or null; run: the
+// kernel's tile body, run(tile, ts).
+template <typename RunTile>
+__device__ __forceinline__ void overlapped_steps(const Inst* __restrict__ insts, const Inst* single,
+                                                 const Tile* __restrict__ tiles, int ntiles, int nsteps, GridBar* bar,
+                                                 unsigned max_polls, const FlowPlan& flow, const RunTile& run) {
   __shared__ long long s_q;
   __shared__ int s_ok;
   __shared__ double s_rho;
   if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < flow.ninst; i += B) flow.step0[i] = (PCONST ? kp.I.st : insts[i].st)->step;
+    for (int i = threadIdx.x; i < flow.ninst; i += blockDim.x) flow.step0[i] = (single ? single->st : insts[i].st)->step;
   }
   if (!grid_barrier(bar, gridDim.x, max_polls, &s_ok)) {
-    if (threadIdx.x == 0) atomicOr(&(PCONST ? kp.I.st : insts[tiles[0].inst].st)->status, STATUS_TIMEOUT);
+    if (threadIdx.x == 0) atomicOr(&(single ? single->st : insts[tiles[0].inst].st)->status, STATUS_TIMEOUT);
     return;
   }
   const long long total = (long long)nsteps * ntiles;
@@ -1623,7 +1433,7 @@ __device__ __forceinline__ void overlapped_steps(const Inst* __restrict__ insts,
     if (q >= total) return;
     const int k = (int)(q / ntiles);
     const Tile tile = tiles[q - (long long)k * ntiles];
-    const Inst& Ii = PCONST ? kp.I : insts[tile.inst];
+    const Inst& Ii = single ? *single : insts[tile.inst];
     const FlowInst& fi = flow.inst ? flow.inst[tile.inst] : flow.single;
     InstState* st = Ii.st;
     const long long step = flow.step0[tile.inst] + k;
@@ -1700,7 +1510,7 @@ __device__ __forceinline__ void overlapped_steps(const Inst* __restrict__ insts,
     ts.local = k == 0 && st->local_read != 0;
     ts.post_open = true;
     ts.rho_avg_prev = s_rho;
-    fused_tile<Real, THERMAL, B, MODE_STEP, FULL, PCONST, INTERIOR>(insts, tile, kp, dyn_smem, sh, ts);
+    run(tile, ts);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();  // the tile's populations are written before its count
@@ -1711,7 +1521,7 @@ __device__ __forceinline__ void overlapped_steps(const Inst* __restrict__ insts,
 }
 
 template <typename Real, bool THERMAL, int B, bool FULL, bool PCONST, bool INTERIOR>
-__global__ void __launch_bounds__(B, (step_min_blocks<Real, B, INTERIOR>()))
+__global__ void __launch_bounds__(B, (step_min_blocks<Real, B>()))
 lbm_persistent_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int ntiles, int nsteps,
                       GridBar* bar, unsigned max_polls, const __grid_constant__ KParams<Real> kp,
                       const __grid_constant__ FlowPlan flow) {
@@ -1723,8 +1533,10 @@ lbm_persistent_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ t
   // from the step's counter, so that the tall bands dispatched first are shared out as they end.
   const bool one_wave = ntiles <= (int)gridDim.x;
   if (!one_wave && flow.enabled) {
-    overlapped_steps<Real, THERMAL, B, FULL, PCONST, INTERIOR>(insts, tiles, ntiles, nsteps, bar, max_polls, kp,
-                                                               flow, dyn_smem, sh);
+    overlapped_steps(insts, PCONST ? &kp.I : nullptr, tiles, ntiles, nsteps, bar, max_polls, flow,
+                     [&](const Tile& tile, const TileStep& ts) {
+                       fused_tile<Real, THERMAL, B, MODE_STEP, FULL, PCONST, INTERIOR>(insts, tile, kp, dyn_smem, sh, ts);
+                     });
     return;
   }
   for (int n = 0; n < nsteps; ++n) {
@@ -1804,15 +1616,19 @@ cudaError_t launch_persistent_cols(bool full, bool interior, const Inst* d_inst,
   if (h_inst) {
     kp.I = *h_inst;
     fill_consts<Real>(kp.C, *h_inst, h_inst->rho_ref);
-    if (interior)
-      return launch_persistent_one<Real, THERMAL, B, false, true, true>(d_inst, d_tiles, ntiles, nsteps, bar,
-                                                                        max_polls, s, kp, flow);
+    if constexpr (sizeof(Real) == 8) {
+      if (interior)
+        return launch_persistent_one<Real, THERMAL, B, false, true, true>(d_inst, d_tiles, ntiles, nsteps, bar,
+                                                                          max_polls, s, kp, flow);
+    }
     return launch_persistent_one<Real, THERMAL, B, false, true, false>(d_inst, d_tiles, ntiles, nsteps, bar,
                                                                        max_polls, s, kp, flow);
   }
-  if (interior)
-    return launch_persistent_one<Real, THERMAL, B, false, false, true>(d_inst, d_tiles, ntiles, nsteps, bar,
-                                                                       max_polls, s, kp, flow);
+  if constexpr (sizeof(Real) == 8) {
+    if (interior)
+      return launch_persistent_one<Real, THERMAL, B, false, false, true>(d_inst, d_tiles, ntiles, nsteps, bar,
+                                                                         max_polls, s, kp, flow);
+  }
   return launch_persistent_one<Real, THERMAL, B, false, false, false>(d_inst, d_tiles, ntiles, nsteps, bar, max_polls,
                                                                       s, kp, flow);
 }
@@ -1820,10 +1636,13 @@ cudaError_t launch_persistent_cols(bool full, bool interior, const Inst* d_inst,
 template <typename Real, bool THERMAL, int B>
 int persistent_resident_cols(bool full, bool interior, bool single) {
   if (full) return persistent_resident<Real, THERMAL, B, true, false, false>();
-  if (single) return interior ? persistent_resident<Real, THERMAL, B, false, true, true>()
-                              : persistent_resident<Real, THERMAL, B, false, true, false>();
-  return interior ? persistent_resident<Real, THERMAL, B, false, false, true>()
-                  : persistent_resident<Real, THERMAL, B, false, false, false>();
+  if constexpr (sizeof(Real) == 8) {
+    if (interior)
+      return single ? persistent_resident<Real, THERMAL, B, false, true, true>()
+                    : persistent_resident<Real, THERMAL, B, false, false, true>();
+  }
+  return single ? persistent_resident<Real, THERMAL, B, false, true, false>()
+                : persistent_resident<Real, THERMAL, B, false, false, false>();
 }
 
 template <typename Real>
@@ -1991,7 +1810,10 @@ int resident_form(int thermal, int cols) {
 
 template <typename Real>
 int resident_precision(int thermal, int cols, bool interior) {
-  return interior ? resident_form<Real, true>(thermal, cols) : resident_form<Real, false>(thermal, cols);
+  if constexpr (sizeof(Real) == 8) {
+    if (interior) return resident_form<Real, true>(thermal, cols);
+  }
+  return resident_form<Real, false>(thermal, cols);
 }
 
 // h_inst: the host copy of the launch's only instance (its constants then travel as a kernel
@@ -2006,10 +1828,14 @@ cudaError_t launch_cols(int mode, bool full, bool interior, const Inst* d_inst, 
         KParams<Real> kp;
         kp.I = *h_inst;
         fill_consts<Real>(kp.C, *h_inst, h_inst->rho_ref);
-        if (interior) return launch_one<Real, THERMAL, B, MODE_STEP, false, true, true>(d_inst, d_tiles, ntiles, s, kp);
+        if constexpr (sizeof(Real) == 8) {
+          if (interior) return launch_one<Real, THERMAL, B, MODE_STEP, false, true, true>(d_inst, d_tiles, ntiles, s, kp);
+        }
         return launch_one<Real, THERMAL, B, MODE_STEP, false, true>(d_inst, d_tiles, ntiles, s, kp);
       }
-      if (interior) return launch_one<Real, THERMAL, B, MODE_STEP, false, false, true>(d_inst, d_tiles, ntiles, s);
+      if constexpr (sizeof(Real) == 8) {
+        if (interior) return launch_one<Real, THERMAL, B, MODE_STEP, false, false, true>(d_inst, d_tiles, ntiles, s);
+      }
       return launch_one<Real, THERMAL, B, MODE_STEP, false>(d_inst, d_tiles, ntiles, s);
     case MODE_FIELDS: return launch_one<Real, THERMAL, B, MODE_FIELDS, true>(d_inst, d_tiles, ntiles, s);
     case MODE_POPS: return launch_one<Real, THERMAL, B, MODE_POPS, true>(d_inst, d_tiles, ntiles, s);

@@ -202,7 +202,7 @@ lbm_tma_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, u
   if (!PCONST) {
     const int* src = reinterpret_cast<const int*>(insts + tile.inst);
     int* dst = reinterpret_cast<int*>(&sI);
-    for (int k = tid; k < (int)(sizeof(Inst) / 4); k += B) dst[k] = src[k];
+    for (int k = tid; k < (int)(offsetof(Inst, strip) / 4); k += B) dst[k] = src[k];
     __syncthreads();
   }
   const Inst& I = PCONST ? kp.I : sI;
@@ -427,7 +427,7 @@ lbm_tma_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, u
 
   // ---------------- per-tile partials into the launch's totals ----------------
   double acc[NPART] = {(double)acc_m, (double)acc_e, (double)acc_h, (double)acc_fi, (double)acc_fo, 0.0, 0.0, 0.0, 0.0};
-  post_partials<B, THERMAL, MODE_STEP>(I, st, tile, acc, sRed, &sLast, step);
+  post_partials<B / 32, THERMAL, MODE_STEP>(I, st, tile, acc, sRed, &sLast, step);
 }
 
 template <bool THERMAL, bool PCONST>
