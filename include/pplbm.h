@@ -286,7 +286,11 @@ int32_t lbm_step_kernel(const lbm_ctx* ctx);
  * the paper's time loop, Sec. 2 and Fig. 2, is the same either way).
  *   LBM_LOOP_LAUNCHES: one step-kernel launch per step.
  *   LBM_LOOP_PERSISTENT: one cooperative launch per call advances all nsteps steps (nsteps >= 2;
- *     a single step is one launch).  Where the step tiling fits in one wave, each CTA keeps
+ *     a single step is one launch).  FP32 lattices with the default tiling and few tiles per SM
+ *     (up to about 300 000 nodes) run all their rows at once, a CTA per tile and a warp per row;
+ *     every CTA keeps its tiles, and a tile waits for the tiles around it and, before the force,
+ *     for the mean density of the step before (reported as LBM_LOOP_PERSISTENT with one tile per
+ *     CTA, as LBM_LOOP_OVERLAPPED with several).  Otherwise, where the step tiling fits in one wave, each CTA keeps
  *     its tile and the CTAs meet at a grid-wide barrier between steps.  Where it needs more
  *     CTAs than are resident, and the geometry is a channel, walls or periodic box, the
  *     launch overlaps consecutive steps (reported as LBM_LOOP_OVERLAPPED): the CTAs draw
@@ -303,7 +307,8 @@ int32_t lbm_step_kernel(const lbm_ctx* ctx);
  *     initialised again (lbm_set_params, lbm_init_fields, lbm_set_populations or
  *     lbm_load_state), and the CUDA context stays usable.  All forms but
  *     LBM_KERNEL_TMA have a persistent form.
- *   LBM_LOOP_AUTO (default): persistent where the step tiling fits in one wave of the
+ *   LBM_LOOP_AUTO (default): persistent where the lattice is small enough for the launch with a
+ *     warp per row (which also takes single steps), where the step tiling fits in one wave of the
  *     persistent kernel (small lattices, whose steps are short enough for the launch gap and
  *     the kernel boundary to count) or where it takes at least two and a half waves and the
  *     launch can overlap the steps, else one launch per step.

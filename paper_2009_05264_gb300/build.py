@@ -20,7 +20,7 @@ OUT_DIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT_DIR, "libpplbm.so")
 BOUNDS_DIR = os.path.join(PKG, "_lib_bounds")
 BOUNDS_LIB = os.path.join(BOUNDS_DIR, "libpplbm.so")
-SOURCES = ["lbm_api.cu", "lbm_batch.cu", "lbm_f32.cu", "lbm_f64.cu", "lbm_strip.cu", "lbm_noalloc.cu", "lbm_probe.cu"]
+SOURCES = ["lbm_api.cu", "lbm_batch.cu", "lbm_f32.cu", "lbm_f64.cu", "lbm_strip.cu", "lbm_flat.cu", "lbm_noalloc.cu", "lbm_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

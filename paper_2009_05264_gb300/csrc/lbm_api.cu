@@ -282,8 +282,15 @@ namespace {
 constexpr int kAuxCols = 128;       // tile width of the field/population readback passes
 constexpr int kAuxRows = 32;
 constexpr int kMinRows = 4;          // smallest band a step tiling may use
-constexpr size_t kAlign = 256;
 constexpr int kMaxDim = 1 << 20;
+
+constexpr size_t kAlign = 256;
+constexpr int kMaxFlatTiles = 1368;  // FLAT_AUTO_ROUNDS tiles on each of three CTAs of 152 SMs
+
+// Barrier status, totals and done counts of a flat launch, cleared together before it.
+size_t flat_state_bytes(int tiles) {
+  return kAlign + sizeof(FlatState) + (size_t)tiles * FLAT_DONE_STRIDE * sizeof(unsigned);
+}
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -292,8 +299,9 @@ struct Layout {
   long long plane;
   size_t pop_bytes;  // one 9-plane buffer
   int max_tiles;
+  int max_flat;      // tiles of the flat launch, at most
   size_t off_f[2], off_g[2], off_rho_prev, off_tmaps, off_inst, off_state, off_sums, off_bar, off_cells, off_step0, off_ring,
-      off_tiles_step, off_tiles_aux, total;
+      off_tiles_step, off_tiles_aux, off_flat, off_tiles_flat, total;
 };
 
 Layout make_layout(int nx, int ny, lbm_precision prec) {
@@ -319,6 +327,9 @@ Layout make_layout(int nx, int ny, lbm_precision prec) {
   L.off_ring = off; off += align_up((size_t)RING * NDIAG * sizeof(double));
   L.off_tiles_step = off; off += align_up((size_t)L.max_tiles * sizeof(Tile));
   L.off_tiles_aux = off; off += align_up((size_t)L.max_tiles * sizeof(Tile));
+  L.max_flat = prec == LBM_FP32 ? (int)std::min<long long>(kMaxFlatTiles, L.max_tiles) : 0;
+  L.off_flat = off; off += align_up(flat_state_bytes(L.max_flat));
+  L.off_tiles_flat = off; off += align_up((size_t)L.max_flat * sizeof(FlatTile));
   L.total = off;
   return L;
 }
@@ -411,9 +422,11 @@ struct lbm_ctx {
   InstState* h_state = nullptr;  // pinned mirror
   int cols = 128, rows = 16;
   BandPlan plan{0, 0, 16};  // the step tiling's bands
+  bool member = false;       // a batch steps it (and plans its own flat launch)
   bool rows_default = true;  // band height chosen by default_band_rows (re-chosen on changes)
   int ntiles_step = 0, ntiles_aux = 0;
   int nopen_step = 0;  // step tiles with an open end (inlet or outlet columns)
+  int flat_tiles = 0, flat_warps = 0, flat_grid = 0;  // the flat launch's tiles, warps per CTA and CTAs (0: none)
   Tile* d_tiles_step = nullptr;
   Tile* d_tiles_aux = nullptr;
   lbm_params params{};
@@ -493,14 +506,41 @@ int step_kernel(const lbm_ctx* c, int cols) {
   return resolve_kernel(c->kernel, c->prec == LBM_FP64, needs_full_step(c->hinst), c->have_tmaps, cols);
 }
 
+// The flat launch's tiles, where the strip kernel runs with the default tiling and the lattice is
+// small enough (FLAT_AUTO_ROUNDS).
+lbm_status plan_flat(lbm_ctx* c) {
+  c->flat_tiles = 0;
+  if (c->member || !c->have_params || !c->rows_default || c->cols != 128 || step_kernel(c, c->cols) != FORM_STRIP) return LBM_OK;
+  int dev = 0, sms = 0, per_sm[22] = {};
+  LBM_CUDA(c, cudaGetDevice(&dev));
+  LBM_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  for (int w = 10; w <= 21; ++w) per_sm[w] = flat_resident_ctas(c->thermal, step_flags(c->hinst), true, w);
+  const int rows = flat_rows({{c->nx, c->ny}}, sms, FLAT_AUTO_ROUNDS, per_sm);
+  if (rows == 0) return LBM_OK;
+  std::vector<FlatTile> t;
+  if (!build_flat_tiles(0, c->nx, c->ny, c->params.geometry, rows, t) || (int)t.size() > c->L.max_flat) return LBM_OK;
+  LBM_CUDA(c, cudaMemcpyAsync(c->base + c->L.off_tiles_flat, t.data(), t.size() * sizeof(FlatTile),
+                              cudaMemcpyHostToDevice, c->stream));
+  LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  c->flat_tiles = (int)t.size();
+  c->flat_warps = rows + 6;
+  c->flat_grid = (int)std::min<long long>(c->flat_tiles, (long long)sms * per_sm[rows + 6]);
+  return LBM_OK;
+}
+
+// Whether step calls take the flat launch: where there is a plan, unless one launch per step is
+// asked for.
+bool use_flat(const lbm_ctx* c) { return c->flat_tiles > 0 && c->loop != LBM_LOOP_LAUNCHES; }
+
 // Re-choose the default tiling for the current kernel, precision and thermal flag.
 lbm_status retile_default(lbm_ctx* c, int cols) {
   const long long slots =
       step_wave_slots(c->prec == LBM_FP64, c->have_params ? c->thermal : 1, cols, step_kernel(c, cols),
                       step_flags(c->hinst));
   const lbm_status s = set_tiling(c, cols, default_band_plan(c->nx, c->ny, cols, slots));
-  if (s == LBM_OK) c->rows_default = true;
-  return s;
+  if (s != LBM_OK) return s;
+  c->rows_default = true;
+  return plan_flat(c);
 }
 
 // Whether a persistent launch of this context may overlap consecutive steps (FlowPlan): the
@@ -657,6 +697,7 @@ lbm_status create_impl(lbm_ctx** out, int32_t nx, int32_t ny, lbm_precision prec
 namespace pplbm {
 Inst lbm_internal_inst(const lbm_ctx* c) { return c->hinst; }
 unsigned long long lbm_internal_params_gen(const lbm_ctx* c) { return c->params_gen; }
+void lbm_internal_set_member(lbm_ctx* c) { c->member = true; }
 }  // namespace pplbm
 
 extern "C" {
@@ -774,6 +815,24 @@ lbm_status lbm_step_async(lbm_ctx* c, int64_t nsteps) {
   if (nsteps < 0) return fail(c, LBM_EINVAL, "nsteps < 0");
   if (!c->have_params) return fail(c, LBM_ESTATE, "lbm_set_params first");
   DeviceGuard g(c->device);
+  if (nsteps >= 1 && use_flat(c)) {
+    char* const base = c->base + c->L.off_flat;
+    GridBar* const bar = reinterpret_cast<GridBar*>(base);
+    FlatState* const fs = reinterpret_cast<FlatState*>(base + kAlign);
+    unsigned* const done = reinterpret_cast<unsigned*>(base + kAlign + sizeof(FlatState));
+    for (int64_t at = 0; at < nsteps;) {
+      const int n = (int)std::min<int64_t>(nsteps - at, FLAT_MAX_STEPS);
+      LBM_CUDA(c, cudaMemsetAsync(base, 0, flat_state_bytes(c->flat_tiles), c->stream));
+      const cudaError_t e = launch_flat(c->thermal, step_flags(c->hinst), c->flat_warps, c->d_inst,
+                                        reinterpret_cast<const FlatTile*>(c->base + c->L.off_tiles_flat),
+                                        c->flat_tiles, c->flat_grid, n, fs, done, bar, c->max_polls, c->stream,
+                                        &c->hinst);
+      if (e != cudaSuccess) return cuda_fail(c, e, "flat kernel launch");
+      ++c->launches;
+      at += n;
+    }
+    return LBM_OK;
+  }
   if (nsteps >= 2 && use_persistent(c)) {
     const int kernel = step_kernel(c, c->cols);
     const int flags = step_flags(c->hinst);
@@ -1043,6 +1102,7 @@ lbm_status lbm_set_kernel(lbm_ctx* c, int32_t kernel) {
   if (kernel < LBM_KERNEL_AUTO || kernel > LBM_KERNEL_INTERIOR)
     return fail(c, LBM_EINVAL, "kernel must be LBM_KERNEL_AUTO, _SCALAR, _PAIRED, _TMA or _INTERIOR");
   c->kernel = kernel;
+  c->flat_tiles = 0;
   if (!c->rows_default) return LBM_OK;
   DeviceGuard g(c->device);
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1067,6 +1127,7 @@ int32_t lbm_step_loop(lbm_ctx* c) {
   if (!c) return -1;
   if (!c->have_params) return c->loop == LBM_LOOP_PERSISTENT ? LBM_LOOP_PERSISTENT : LBM_LOOP_LAUNCHES;
   DeviceGuard g(c->device);
+  if (use_flat(c)) return c->flat_tiles > c->flat_grid ? LBM_LOOP_OVERLAPPED : LBM_LOOP_PERSISTENT;
   if (!use_persistent(c)) return LBM_LOOP_LAUNCHES;
   return overlapped(c) ? LBM_LOOP_OVERLAPPED : LBM_LOOP_PERSISTENT;
 }
@@ -1155,7 +1216,10 @@ lbm_status lbm_set_tiling(lbm_ctx* c, int32_t cols, int32_t rows) {
   rows = std::min(rows, c->ny);
   if (rows < kMinRows && rows < c->ny) return fail(c, LBM_EINVAL, "rows must be >= 4 (or the full height)");
   const lbm_status s = set_tiling(c, cols, BandPlan{0, 0, rows});
-  if (s == LBM_OK) c->rows_default = false;
+  if (s == LBM_OK) {
+    c->rows_default = false;
+    c->flat_tiles = 0;
+  }
   return s;
 }
 

@@ -59,6 +59,12 @@ struct lbm_batch {
   FlowInst* d_flow = nullptr;
   long long* d_step0 = nullptr;
   unsigned long long* d_cells = nullptr;
+  // flat launch (lbm_flat.cuh): its tiles, and per launch the barrier status, the members' totals and
+  // the tiles' done counts (one block, cleared before the launch)
+  FlatTile* d_flat_tiles = nullptr;
+  char* d_flat_state = nullptr;
+  size_t cap_flat = 0, cap_flat_state = 0;
+  int flat_tiles = 0, flat_warps = 0, flat_grid = 0;  // 0 tiles: none
   bool flow_ok = false;  // every member may run overlapped (no pool, distinct inlet and outlet)
   std::string err;
 };
@@ -90,6 +96,51 @@ BandPlan member_plan(const lbm_batch* b, int nx, int ny, long long slots, double
   if (b->rows > 0) return BandPlan{0, 0, std::max(1, std::min(b->rows, ny))};
   const long long member_slots = std::max<long long>(1, (long long)(slots * share + 0.5));
   return default_band_plan(nx, ny, b->cols, member_slots);
+}
+
+constexpr size_t kFlatHead = 256;  // the GridBar, with the rest aligned behind it
+size_t flat_state_bytes(size_t insts, size_t tiles) {
+  return kFlatHead + insts * sizeof(FlatState) + tiles * FLAT_DONE_STRIDE * sizeof(unsigned);
+}
+
+// The flat launch's tiles over all members, where the strip kernel runs with the default tiling and
+// the members together are small enough (FLAT_BATCH_ROUNDS).
+lbm_status plan_flat(lbm_batch* b, const std::vector<Inst>& insts) {
+  b->flat_tiles = 0;
+  if (insts.empty() || b->launch_kernel != FORM_STRIP || b->rows != 0 || b->cols != 128) return LBM_OK;
+  int dev = 0, sms = 0, per_sm[22] = {};
+  LBM_BCUDA(b, cudaGetDevice(&dev));
+  LBM_BCUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  for (int w = 10; w <= 21; ++w) per_sm[w] = flat_resident_ctas(b->thermal, b->flags, false, w);
+  std::vector<FlatSize> sizes;
+  for (const Inst& I : insts) sizes.push_back({I.nx, I.ny});
+  const int rows = flat_rows(sizes, sms, FLAT_BATCH_ROUNDS, per_sm);
+  if (rows == 0) return LBM_OK;
+  std::vector<FlatTile> t;
+  for (size_t i = 0; i < insts.size(); ++i)
+    if (!build_flat_tiles((int)i, insts[i].nx, insts[i].ny, insts[i].geometry, rows, t)) return LBM_OK;
+  if (t.size() > b->cap_flat) {
+    if (b->d_flat_tiles) cudaFree(b->d_flat_tiles);
+    b->d_flat_tiles = nullptr;
+    b->cap_flat = 0;
+    if (cudaMalloc(&b->d_flat_tiles, t.size() * sizeof(FlatTile)) != cudaSuccess)
+      return bfail(b, LBM_ENOMEM, "flat tile table");
+    b->cap_flat = t.size();
+  }
+  const size_t bytes = flat_state_bytes(insts.size(), t.size());
+  if (bytes > b->cap_flat_state) {
+    if (b->d_flat_state) cudaFree(b->d_flat_state);
+    b->d_flat_state = nullptr;
+    b->cap_flat_state = 0;
+    if (cudaMalloc(&b->d_flat_state, bytes) != cudaSuccess) return bfail(b, LBM_ENOMEM, "flat launch state");
+    b->cap_flat_state = bytes;
+  }
+  LBM_BCUDA(b, cudaMemcpyAsync(b->d_flat_tiles, t.data(), t.size() * sizeof(FlatTile), cudaMemcpyHostToDevice, b->stream));
+  LBM_BCUDA(b, cudaStreamSynchronize(b->stream));
+  b->flat_tiles = (int)t.size();
+  b->flat_warps = rows + 6;
+  b->flat_grid = (int)std::min<long long>(b->flat_tiles, (long long)sms * per_sm[rows + 6]);
+  return LBM_OK;
 }
 
 // Upload the descriptors and the concatenated tile table of the active members.
@@ -200,6 +251,8 @@ lbm_status rebuild(lbm_batch* b) {
   b->launch_kernel = launch_kernel;
   b->flags = flags;
   drop_graph(b);
+  const lbm_status s = plan_flat(b, insts);
+  if (s != LBM_OK) return s;
   b->dirty = false;
   return LBM_OK;
 }
@@ -256,6 +309,27 @@ lbm_status launch_persistent_steps(lbm_batch* b, int64_t nsteps) {
                                    b->d_tiles, b->ntiles, n, b->d_bar, b->max_polls, b->stream, nullptr, flow));
     ++b->launches;
     done += n;
+  }
+  return LBM_OK;
+}
+
+// Whether step calls take the flat launch: where there is a plan, unless one launch per step is
+// asked for.
+bool batch_flat(const lbm_batch* b) { return b->flat_tiles > 0 && b->loop != LBM_LOOP_LAUNCHES; }
+
+lbm_status launch_flat_steps(lbm_batch* b, int64_t nsteps) {
+  size_t ninst = 0;
+  for (const Member& m : b->slots) ninst += m.ctx != nullptr;
+  GridBar* const bar = reinterpret_cast<GridBar*>(b->d_flat_state);
+  FlatState* const fs = reinterpret_cast<FlatState*>(b->d_flat_state + kFlatHead);
+  unsigned* const done = reinterpret_cast<unsigned*>(b->d_flat_state + kFlatHead + ninst * sizeof(FlatState));
+  for (int64_t at = 0; at < nsteps;) {
+    const int n = (int)std::min<int64_t>(nsteps - at, FLAT_MAX_STEPS);
+    LBM_BCUDA(b, cudaMemsetAsync(b->d_flat_state, 0, flat_state_bytes(ninst, b->flat_tiles), b->stream));
+    LBM_BCUDA(b, launch_flat(b->thermal, b->flags, b->flat_warps, b->d_insts, b->d_flat_tiles, b->flat_tiles,
+                             b->flat_grid, n, fs, done, bar, b->max_polls, b->stream, nullptr));
+    ++b->launches;
+    at += n;
   }
   return LBM_OK;
 }
@@ -324,6 +398,7 @@ lbm_status lbm_batch_add(lbm_batch* b, int32_t nx, int32_t ny, const lbm_params*
   lbm_ctx* c = nullptr;
   lbm_status s = lbm_create(&c, nx, ny, b->prec, b->device, b->stream);
   if (s != LBM_OK) return bfail(b, s, "member creation failed");
+  lbm_internal_set_member(c);
   s = lbm_set_params(c, p);
   if (s != LBM_OK) {
     b->err = lbm_last_error(c);
@@ -406,7 +481,9 @@ lbm_status lbm_batch_step_async(lbm_batch* b, int64_t nsteps) {
   for (const Member& m : b->slots)  // a member's parameters or state were replaced directly
     if (m.ctx && m.gen != lbm_internal_params_gen(m.ctx)) b->dirty = true;
   if (b->dirty) s = rebuild(b);
-  if (s == LBM_OK && b->ntiles > 0 && nsteps >= 2 && batch_persistent(b)) {
+  if (s == LBM_OK && b->ntiles > 0 && nsteps >= 1 && batch_flat(b)) {
+    s = launch_flat_steps(b, nsteps);
+  } else if (s == LBM_OK && b->ntiles > 0 && nsteps >= 2 && batch_persistent(b)) {
     s = launch_persistent_steps(b, nsteps);
   } else if (s == LBM_OK && b->ntiles > 0) {
     int64_t left = nsteps;
@@ -438,7 +515,8 @@ int32_t lbm_batch_step_loop(lbm_batch* b) {
   cudaSetDevice(b->device);
   int32_t out = -1;
   if (!b->dirty || rebuild(b) == LBM_OK)
-    out = !batch_persistent(b) ? LBM_LOOP_LAUNCHES : (batch_overlapped(b) ? LBM_LOOP_OVERLAPPED : LBM_LOOP_PERSISTENT);
+    out = batch_flat(b) ? (b->flat_tiles > b->flat_grid ? LBM_LOOP_OVERLAPPED : LBM_LOOP_PERSISTENT)
+          : !batch_persistent(b) ? LBM_LOOP_LAUNCHES : (batch_overlapped(b) ? LBM_LOOP_OVERLAPPED : LBM_LOOP_PERSISTENT);
   if (prev >= 0) cudaSetDevice(prev);
   return out;
 }
@@ -540,6 +618,8 @@ lbm_status lbm_batch_destroy(lbm_batch* b) {
   if (b->d_flow) cudaFree(b->d_flow);
   if (b->d_step0) cudaFree(b->d_step0);
   if (b->d_cells) cudaFree(b->d_cells);
+  if (b->d_flat_tiles) cudaFree(b->d_flat_tiles);
+  if (b->d_flat_state) cudaFree(b->d_flat_state);
   if (b->own_stream) cudaStreamDestroy(b->stream);
   if (prev >= 0) cudaSetDevice(prev);
   delete b;

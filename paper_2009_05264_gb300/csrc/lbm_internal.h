@@ -5,6 +5,8 @@
 #include <nvtx3/nvToolsExt.h>  // header-only: ranges cost nothing unless a profiler is attached
 #include <stdint.h>
 
+#include <vector>
+
 #include "pplbm.h"
 
 namespace pplbm {
@@ -272,6 +274,33 @@ struct FlowPlan {
   unsigned long long* cell_done;   // per tile position (cell_base + band * strips + strip): steps
                                    // of this launch it has finished (zeroed before the launch)
 };
+// Flat persistent launch (lbm_flat.cuh): a CTA per tile, a warp per row, every CTA owning its
+// tiles for all the steps.  A tile of step s waits for the tiles around it (deps: what its pulls
+// read) to have finished step s - 1, and for the mass totals of step s - 1 to be complete.
+constexpr int FLAT_MAX_DEPS = 25;
+struct FlatTile {
+  short inst, wout;            // output columns [x0, x0 + wout), rows [y0, y0 + rows)
+  int x0, y0, rows;
+  int ntiles;                  // tiles of the instance
+  int ndeps;
+  int deps[FLAT_MAX_DEPS];     // positions in the launch's tile table
+  unsigned char dep_rows[FLAT_MAX_DEPS + 3];  // rows of those tiles: each adds one count per row and step
+};
+// Per instance, zeroed before the launch: step s uses slot s % 4 of the totals, of the pressure
+// probes and of the counts of tiles; the last tile of step s clears the slot of step s - 1, which
+// every tile has read by then.  What different warps poll and add to lies on different cache lines.
+struct __align__(128) FlatSlot {
+  unsigned int count;                           // tiles that have added their mass
+  unsigned int pad0[31];
+  unsigned long long sums[16];                  // NPART totals, the mass first
+  unsigned int complete;                        // tiles that have added all their sums
+  unsigned int pad1[31];
+  double probe[16];
+};
+struct FlatState {
+  FlatSlot slot[4];
+};
+constexpr int FLAT_DONE_STRIDE = 32;  // a tile's count of finished rows, one per cache line
 struct GridBar {
   unsigned int count, gen, status, pad;
   unsigned int next[2];
@@ -309,6 +338,27 @@ inline bool general_tile(const Tile& t) { return !t.interior; }
 cudaError_t launch_lbm(int fp64, int thermal, int cols, int mode, int kernel, int flags, const Inst* d_inst,
                        const Tile* d_tiles, int ntiles, cudaStream_t s, const Inst* h_inst = nullptr,
                        unsigned max_polls = 0);
+// nsteps steps of the flat FP32 kernel in one cooperative launch of `grid` CTAs of `warps` warps over
+// the tiles of build_flat_tiles (tile i on CTA i % grid); fstate (per instance) and done (per
+// tile) zeroed.
+cudaError_t launch_flat(int thermal, int flags, int warps, const Inst* d_inst, const FlatTile* d_tiles, int ntiles,
+                        int grid, int nsteps, FlatState* fstate, unsigned* done, GridBar* bar, unsigned max_polls,
+                        cudaStream_t s, const Inst* h_inst);
+int flat_resident_ctas(int thermal, int flags, bool single, int warps);
+struct FlatSize {
+  int nx, ny;
+};
+bool build_flat_tiles(int inst, int nx, int ny, int geometry, int rows, std::vector<FlatTile>& out);
+// per_sm_by_warps: resident CTAs per SM by warps per CTA (indices 0 .. 21).
+int flat_rows(const std::vector<FlatSize>& sizes, int sms, int max_rounds, const int* per_sm_by_warps);
+constexpr int FLAT_MAX_STEPS = 1 << 27;  // of a launch: steps times rows stay below 2^32
+constexpr double FLAT_ROUND_COST = 10.0;  // in warps
+// Rounds (tiles per CTA) up to which the flat launch is taken.  A round costs about 6 us whatever the
+// size, the strip kernel no less than 20 us a step: 1500 x 150 (2 rounds) 12.7 against 20.1 us,
+// 1800 x 160 (3) 17.0 against 19.9, 2000 x 200 (4) 24.2 against 24.6, 2500 x 220 (5) 31.3 against
+// 26.7.  A batch's strip kernel reads its constants from shared memory and is a little slower:
+// four 128 x 512 pools (3 rounds) 21.5 against 28.9 us, six (5) 34.1 against 31.8.
+constexpr int FLAT_AUTO_ROUNDS = 3, FLAT_BATCH_ROUNDS = 4;
 // nsteps steps of the step kernel in one cooperative launch (tiles drawn dynamically from a
 // counter, a bounded grid barrier between steps; MODE_STEP only).  grid <= resident CTAs of
 // the device; bar: zeroed GridBar in device memory.
@@ -401,5 +451,7 @@ int resident_ctas_f64(int thermal, int cols, int kernel);
 Inst lbm_internal_inst(const lbm_ctx* c);
 // Changes whenever the context's descriptor is rewritten (parameters or a loaded state).
 unsigned long long lbm_internal_params_gen(const lbm_ctx* c);
+// Marks a context as a batch's member (before its parameters are set).
+void lbm_internal_set_member(lbm_ctx* c);
 
 }  // namespace pplbm
