@@ -218,9 +218,9 @@ __device__ __forceinline__ bool flat_row(const Inst& I, const StripTile& t, cons
     if (out) {
       if (EDGE && L.channel) {
         float fi = 0.0f, fo = 0.0f;
-        if (L.inl_a && L.out_a) fi = o.rho.x * o.uax.x;
-        if (L.outl_a && L.out_a) fo = o.rho.x * o.uax.x;
-        if (L.outl_b && L.out_b) fo = o.rho.y * o.uax.y;
+        if (L.inl_a && L.out_a) fi = __fmaf_rn(0.5f, o.Fx.x, n.jx.x);  // rho u_act = j + F / 2
+        if (L.outl_a && L.out_a) fo = __fmaf_rn(0.5f, o.Fx.x, n.jx.x);
+        if (L.outl_b && L.out_b) fo = __fmaf_rn(0.5f, o.Fx.y, n.jx.y);
         fi = warp_sum(fi);  // one lane's value: exact
         fo = warp_sum(fo);
         if (L.lane == 0) {

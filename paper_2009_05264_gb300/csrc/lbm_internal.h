@@ -85,6 +85,8 @@ struct KConst {
   // products of the constants above, formed once (host doubles): R / (1 - b rho_ref),
   // a / D(rho_ref), 2 b rho_ref, -kappa / sqrt(Tc), a rho_ref^2 / D(rho_ref)
   Real R_u1r, a_Dr, twob_rr, nk_sTc, a_rr2_Dr;
+  // FP64 step: G / 4, 1 + kappa, psi_scale R, psi_scale a, psi_scale / 3, R / c_v, -a kappa / (sqrt(Tc) c_v)
+  Real Ghh, kappa1, R_ps, a_ps, ps_3, R_cv, ank_cv;
 };
 
 // Constants of the packed step, each held twice so that a packed instruction takes it as one
@@ -204,6 +206,13 @@ __host__ __device__ inline void fill_consts(KConst<Real>& c, const Inst& I, doub
   c.twob_rr = Real(I.twob_rr);
   c.nk_sTc = Real(I.nk_sTc);
   c.a_rr2_Dr = Real(I.a_rr2_Dr);
+  c.Ghh = Real(0.5 * I.Ghalf);
+  c.kappa1 = Real(1.0 + I.kappa);
+  c.R_ps = Real(I.R * I.psi_scale);
+  c.a_ps = Real(I.a * I.psi_scale);
+  c.ps_3 = Real(I.psi_scale * (1.0 / 3.0));
+  c.R_cv = Real(I.R * I.inv_cv);
+  c.ank_cv = Real(I.a * I.nk_sTc * I.inv_cv);
 }
 
 __host__ __device__ inline float2 pair_of(double v) { return make_float2((float)v, (float)v); }

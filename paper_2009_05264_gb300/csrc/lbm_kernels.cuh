@@ -92,34 +92,57 @@ __device__ inline Real& bounds_sink() {
 __device__ __forceinline__ constexpr bool idx_ok(InstState*, long long, long long) { return true; }
 #endif
 
+// Products and multiply-adds that the compiler neither splits nor fuses, so that the force and the
+// f collision round alike in every kernel form.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mad_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mad_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // Reciprocal and reciprocal square root.  FP32: MUFU approximations (about 2 ulp).  FP64: the
-// PTX approximations rcp.approx / rsqrt.approx (about 23 correct bits) refined by two
-// Newton-Raphson steps on f(y) = 1/y - x and f(y) = 1/y^2 - x (each step squares the relative
-// error), which ends within a few ulp of the correctly rounded result in fewer FP64
-// instructions than an IEEE division or square root on this GPU's narrow FP64 pipe; inputs are
-// positive normal numbers here (densities, temperatures, psi radicands).
+// PTX approximations rcp.approx / rsqrt.approx (about 22 correct bits) refined by one
+// third-order step (Householder's method on f(y) = 1/y - x and f(y) = 1/y^2 - x): with e the
+// relative error of x y, or of x y^2, 1/x = y (1 + e + e^2 + ...) and
+// 1/sqrt(x) = y (1 + e/2 + 3/8 e^2 + ...), cut after e^2, which leaves e^3 < 2^-60.  Three and
+// five FP64 instructions against the four and eight of two Newton-Raphson steps, within a few
+// ulp of the correctly rounded result; inputs are positive normal numbers here (densities,
+// temperatures, psi radicands).
 __device__ __forceinline__ float fast_rcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double fast_rcp(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);  // relative error of y
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 __device__ __forceinline__ float fast_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double fast_rsqrt(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(x));
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double e = fma(-x, y * y, 1.0);  // 1 - x y^2
-    y = fma(0.5 * y, e, y);
-  }
-  return y;
+  const double e = fma(-x, y * y, 1.0);
+  return fma(y, e * fma(0.375, e, 0.5), y);
 }
 __device__ __forceinline__ float fast_sqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
-__device__ __forceinline__ double fast_sqrt(double x) { return x > 0.0 ? x * fast_rsqrt(x) : 0.0; }
+// x > 0, x >= 0 and |x| < inf of a double (false for NaN), from its upper word: a comparison of
+// doubles takes the FP64 pipe, this the integer one.  (Below 2^-1042 a positive x counts as 0.)
+__device__ __forceinline__ bool is_positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool is_positive(double x) { return (unsigned)(__double2hiint(x) - 1) < 0x7ff00000u; }
+__device__ __forceinline__ bool is_nonnegative(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool is_nonnegative(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  return hi <= 0x7ff00000u || hi == 0x80000000u;
+}
+__device__ __forceinline__ bool is_finite(float x) { return fabsf(x) < INFINITY; }
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x7ff00000; }
+// The third-order step on s = x y itself, its residual x - s^2 exact to rounding: no more
+// instructions than x times 1/sqrt(x), and one rounding instead of two.
+__device__ __forceinline__ double fast_sqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(x));
+  const double s = x * y;
+  const double d = fma(-s, s, x) * y;
+  const double r = fma(d, fma(0.375, d * y, 0.5), s);
+  return is_positive(x) ? r : 0.0;
+}
 
 // Asynchronous global -> shared copies of one element (cp.async, Ampere and later).
 __device__ __forceinline__ void cp_async_elem(float* smem, const float* gmem) {
@@ -151,7 +174,7 @@ __host__ __device__ constexpr int out_cols() { return B - 8; }
 
 template <typename Real, bool THERMAL, int B>
 constexpr size_t fused_smem_bytes() {
-  return sizeof(Real) * (size_t)(B - 4) * (9 * F_SLOTS + (THERMAL ? 9 * G_SLOTS : 0) + 9);
+  return sizeof(Real) * (size_t)(B - 4) * (9 * F_SLOTS + (THERMAL ? 9 * G_SLOTS : 0) + 7);
 }
 
 // Rows the interior path stages ahead of the row it computes (its rings hold f of rows
@@ -163,7 +186,7 @@ constexpr int FI_SLOTS = 2 + LOOKAHEAD;
 constexpr int GI_SLOTS = 3 + LOOKAHEAD;
 template <typename Real, bool THERMAL, int B>
 constexpr size_t interior_smem_bytes() {
-  return sizeof(Real) * (size_t)(B - 4) * (9 * FI_SLOTS + (THERMAL ? 9 * GI_SLOTS : 0) + 9);
+  return sizeof(Real) * (size_t)(B - 4) * (9 * FI_SLOTS + (THERMAL ? 9 * GI_SLOTS : 0) + 7);
 }
 // Dynamic shared memory of a step-kernel instantiation (the interior path's layout is larger).
 template <typename Real, bool THERMAL, int B, bool INTERIOR>
@@ -306,11 +329,11 @@ __device__ __forceinline__ void boundary_fill(Real (&fc)[9], Real (&gc)[9], cons
 // Macroscopic state of one node (compute precision; deviations from the references).
 template <typename Real>
 struct NodeState {
-  Real rho, drho, ux, uy, T, dT, coef;  // coef = T (1 - (dp/dT)_rho / (rho c_v)) of the source
+  Real rho, drho, jx, jy, T, dT, coef;  // j: momentum; coef = T (1 - (dp/dT)_rho / (rho c_v)) of the source
   Real inv_rho;                          // 1 / rho
   Real hmc;                              // Hazi-Markus form: T (dp/dT)_rho / (rho^2 c_v); coef is then T
   Real dpsi;                             // psi - psi_ref (psi itself in FP64)
-  Real p;                                // EOS pressure (diagnostics)
+  Real rad;                              // FP64: psi^2; FP32: psi^2 - psi_ref^2 (see node_pressure)
   bool bad;                              // outside the EOS domain
 };
 
@@ -318,6 +341,13 @@ struct NodeState {
 // (dp/dT)_rho of one node.  In FP32 psi is evaluated as psi - psi_ref from exact
 // difference forms of Eq. 12 in rho - rho_ref and T - T_ref, so that neighbour
 // differences in the force keep their low-order bits.
+//
+// FP64: the pipe issues one warp instruction per 64 cycles and SM quarter, and every large
+// lattice's step is bound by it, so the forms are chosen for their count.  With
+// om = 1 - b rho, D = 1 + 2 b rho - (b rho)^2 = 2 - om^2 and sa = sqrt(alpha),
+//   psi^2 = s (p - rho / 3) = rho (s R T / om - s a (sa^2 rho / D) - s / 3),
+//   1 - (dp/dT)_rho / (rho c_v) = 1 - R / (om c_v) + a k / c_v (sa rho / D) / sqrt(T),
+// k = -kappa / sqrt(Tc), the products of constants formed once.
 template <typename Real, bool THERMAL>
 __device__ __forceinline__ NodeState<Real> node_state(const Real (&fc)[9], const Real (&gc)[9],
                                                       const KConst<Real>& C, bool multiphase, bool hazi = false) {
@@ -325,15 +355,14 @@ __device__ __forceinline__ NodeState<Real> node_state(const Real (&fc)[9], const
   o.hmc = Real(0);
   const Real rho_ref = C.rho_ref;
   Real sum_g = Real(0);
-  o.drho = ((fc[0] + fc[1]) + (fc[2] + fc[3])) + ((fc[4] + fc[5]) + (fc[6] + fc[7])) + fc[8];
+  const Real p56 = fc[5] + fc[6], p78 = fc[7] + fc[8];
+  o.drho = ((fc[0] + (fc[1] + fc[3])) + (fc[2] + fc[4])) + (p56 + p78);
   if (THERMAL) sum_g = ((gc[0] + gc[1]) + (gc[2] + gc[3])) + ((gc[4] + gc[5]) + (gc[6] + gc[7])) + gc[8];
   o.rho = rho_ref + o.drho;
-  const Real jx = (fc[1] - fc[3]) + (fc[5] - fc[6]) + (fc[8] - fc[7]);
-  const Real jy = (fc[2] - fc[4]) + (fc[5] + fc[6]) - (fc[7] + fc[8]);
+  o.jx = (fc[1] - fc[3]) + ((fc[5] - fc[6]) + (fc[8] - fc[7]));
+  o.jy = (fc[2] - fc[4]) + (p56 - p78);
   const Real inv_rho = fast_rcp(o.rho);
   o.inv_rho = inv_rho;
-  o.ux = jx * inv_rho;
-  o.uy = jy * inv_rho;
   if (THERMAL) {
     o.dT = sum_g;
     o.T = C.T_ref + o.dT;
@@ -342,28 +371,29 @@ __device__ __forceinline__ NodeState<Real> node_state(const Real (&fc)[9], const
     o.T = C.T0;
   }
   o.dpsi = Real(0);
-  o.p = o.rho * Real(1.0 / 3.0);
+  o.rad = Real(0);
   o.coef = Real(0);
-  Real dpdT = Real(0);
-  bool bad = !(o.rho > Real(0));
+  Real te = Real(0);  // (dp/dT)_rho / (rho c_v)
+  Real cf = Real(1);  // 1 - te
+  bool bad = !is_positive(o.rho);
   if (multiphase) {
-    const Real pa = C.a, pb = C.b, pR = C.R, kappa = C.kappa, inv_sqrtTc = C.inv_sqrtTc;
     const Real rho_c = o.rho, drho_c = o.drho, T_c = o.T, dT_c = o.dT;
-    const Real br = pb * rho_c;
-    const Real inv1 = fast_rcp(Real(1) - br);
-    const Real invD = fast_rcp(Real(1) + br * (Real(2) - br));
-    const Real rr_den = rho_c * rho_c * invD;
-    Real alpha, sa = Real(0), inv_sT = Real(0), sT = Real(0);
-    if (THERMAL) {
-      inv_sT = fast_rsqrt(T_c);
-      sT = T_c * inv_sT;
-      sa = Real(1) + kappa * (Real(1) - sT * inv_sqrtTc);
-      alpha = sa * sa;
-    } else {
-      alpha = C.alpha0;
-    }
-    Real rad;
+    const Real om = Real(1) - C.b * rho_c;
+    const Real inv1 = fast_rcp(om);
+    const Real invD = fast_rcp(Real(2) - om * om);
+    Real sa = Real(0), inv_sT = Real(0), rad;
     if (sizeof(Real) == 4) {
+      const Real pR = C.R, pa = C.a, kappa = C.kappa;
+      const Real rr_den = rho_c * rho_c * invD;
+      Real alpha, sT = Real(0);
+      if (THERMAL) {
+        inv_sT = fast_rsqrt(T_c);
+        sT = T_c * inv_sT;
+        sa = Real(1) + kappa * (Real(1) - sT * C.inv_sqrtTc);
+        alpha = sa * sa;
+      } else {
+        alpha = C.alpha0;
+      }
       const Real rr = rho_ref;
       // R (rho T / (1 - b rho) - rho_ref T_ref / (1 - b rho_ref)) and the attraction term's
       // difference, as exact difference forms in drho = rho - rho_ref and dT = T - T_ref
@@ -372,56 +402,88 @@ __device__ __forceinline__ NodeState<Real> node_state(const Real (&fc)[9], const
       if (THERMAL) {
         const Real dsa = C.nk_sTc * dT_c * fast_rcp(sT + C.sqrtT_r);
         dB += C.a_rr2_Dr * dsa * (sa + C.sa_r);
+        const Real dalpha = C.nk_sTc * sa * inv_sT;  // d alpha / dT = -kappa sqrt(alpha) / sqrt(T Tc)
+        te = (rho_c * pR * inv1 - pa * dalpha * rr_den) * inv_rho * C.inv_cv;
+        cf = Real(1) - te;
       }
-      const Real dp = dA - dB;
-      const Real drad = (dp - drho_c * Real(1.0 / 3.0)) * C.psi_scale;
+      const Real drad = (dA - dB - drho_c * Real(1.0 / 3.0)) * C.psi_scale;
+      o.rad = drad;
       rad = C.rad_ref + drad;
       const Real psi = fast_sqrt(fmax(rad, Real(0)));
       const Real den = psi + C.psi_ref;
       o.dpsi = den > Real(0) ? drad * fast_rcp(den) : Real(0);
-      o.p = C.p_ref + dp;
     } else {
-      o.p = rho_c * pR * T_c * inv1 - pa * alpha * rr_den;
-      rad = (o.p - rho_c * Real(1.0 / 3.0)) * C.psi_scale;
-      o.dpsi = fast_sqrt(fmax(rad, Real(0)));
+      const Real q = rho_c * invD;
+      Real v;  // alpha rho / D
+      if (THERMAL) {
+        inv_sT = fast_rsqrt(T_c);
+        sa = C.nk_sTc * (T_c * inv_sT) + C.kappa1;
+        const Real u = sa * q;
+        v = sa * u;
+        cf = Real(1) - C.R_cv * inv1;
+        cf = C.ank_cv * (u * inv_sT) + cf;
+      } else {
+        v = C.alpha0 * q;
+      }
+      rad = rho_c * (C.R_ps * (T_c * inv1) - (C.a_ps * v + C.ps_3));
+      o.rad = rad;
+      o.dpsi = fast_sqrt(rad);
+      if (THERMAL && hazi) te = Real(1) - cf;
     }
-    bad = bad || !(br < Real(1)) || !(rad >= Real(0));
-    if (THERMAL) {
-      const Real dalpha = C.nk_sTc * sa * inv_sT;  // d alpha / dT = -kappa sqrt(alpha) / sqrt(T Tc)
-      dpdT = rho_c * pR * inv1 - pa * dalpha * rr_den;
-    }
+    bad = bad || !is_positive(om) || !is_nonnegative(rad);
   }
   if (THERMAL) {
-    bad = bad || !isfinite(o.T);
+    bad = bad || !is_finite(o.T);
     if (hazi) {  // first Eq. 19: T div u + T (dp/dT)_rho / (rho^2 c_v) drho/dt
       o.coef = o.T;
-      o.hmc = o.T * dpdT * inv_rho * inv_rho * C.inv_cv;
+      o.hmc = o.T * te * inv_rho;
     } else {     // second Eq. 19
-      o.coef = o.T * (Real(1) - dpdT * inv_rho * C.inv_cv);
+      o.coef = o.T * cf;
     }
   }
   o.bad = bad;
   return o;
 }
+// EOS pressure of a node (Eq. 12; rho / 3 without the multiphase force).
+template <typename Real>
+__device__ __forceinline__ double node_pressure(const NodeState<Real>& n, const KConst<Real>& C, bool multiphase) {
+  if (!multiphase) return (double)(n.rho * Real(1.0 / 3.0));
+  if (sizeof(Real) == 4) return (double)(C.p_ref + (n.rad / C.psi_scale + n.drho * Real(1.0 / 3.0)));
+  return (double)(n.rad / C.psi_scale + n.rho * Real(1.0 / 3.0));
+}
+
+// psi - psi_ref of one row at a node: the node's own, east minus west and east plus west.
+template <typename Real>
+struct PsiLine {
+  Real c, d, s;
+};
+template <typename Real>
+__device__ __forceinline__ PsiLine<Real> psi_line(Real c, Real e, Real w) {
+  return PsiLine<Real>{c, e - w, e + w};
+}
 
 // Interaction force of Eqs. 9, 10, 14, 15 from the neighbours' d = psi - psi_ref
 // (d = 0 for solid neighbours).  With psi = psi_ref + d the beta-mixed sums reduce to
 // F = -(psi_ref + beta d_c) t1 - (1 - beta)/2 t2, t1 = sum G_i d_i c_i,
-// t2 = sum G_i d_i^2 c_i, plus the wall rows' reference parts with Eq. 15.
+// t2 = sum G_i d_i^2 c_i, plus the wall rows' reference parts with Eq. 15.  The squares are
+// taken as products of sums and differences; the diagonal part of t2y is
+// Gh (E_N^2 + W_N^2 - E_S^2 - W_S^2) = Gh / 2 [(s_N - s_S)(s_N + s_S) + (d_N - d_S)(d_N + d_S)].
 template <typename Real>
-__device__ __forceinline__ void sc_force(Real dc, Real dE, Real dW, Real dN, Real dNE, Real dNW, Real dS, Real dSE,
-                                         Real dSW, bool sol_m, bool sol_p, const KConst<Real>& C, Real& Fx,
-                                         Real& Fy) {
+__device__ __forceinline__ void sc_force(const PsiLine<Real>& N, const PsiLine<Real>& M, const PsiLine<Real>& S,
+                                         bool sol_m, bool sol_p, const KConst<Real>& C, Real& Fx, Real& Fy) {
   const Real G2 = C.G2, Gh = C.Gh;
-  const Real t1x = G2 * (dE - dW) + Gh * ((dNE - dNW) + (dSE - dSW));
-  const Real t1y = G2 * (dN - dS) + Gh * ((dNE + dNW) - (dSE + dSW));
-  const Real t2x = G2 * (dE - dW) * (dE + dW) + Gh * ((dNE - dNW) * (dNE + dNW) + (dSE - dSW) * (dSE + dSW));
-  const Real t2y = G2 * (dN - dS) * (dN + dS) + Gh * ((dNE - dSE) * (dNE + dSE) + (dNW - dSW) * (dNW + dSW));
-  const Real lead = C.psi_ref + C.beta * dc;
-  Fx = -lead * t1x - C.mix * t2x;
-  Fy = -lead * t1y - C.mix * t2y;
-  if (sol_m) Fy += C.wall0 + dc * C.wall1;
-  if (sol_p) Fy -= C.wall0 + dc * C.wall1;
+  const Real dsum = N.d + S.d, gd = mul_rn(G2, M.d);
+  const Real cdif = N.c - S.c, sdif = N.s - S.s, gc = mul_rn(G2, cdif);
+  const Real t1x = mad_rn(Gh, dsum, gd);
+  const Real t1y = mad_rn(Gh, sdif, gc);
+  const Real t2x = mad_rn(gd, M.s, mul_rn(Gh, mad_rn(N.d, N.s, mul_rn(S.d, S.s))));
+  const Real m = mad_rn(sdif, N.s + S.s, mul_rn(N.d - S.d, dsum));
+  const Real t2y = mad_rn(gc, N.c + S.c, mul_rn(C.Ghh, m));
+  const Real nlead = mad_rn(-C.beta, M.c, -C.psi_ref);
+  Fx = mad_rn(nlead, t1x, mul_rn(-C.mix, t2x));
+  Fy = mad_rn(nlead, t1y, mul_rn(-C.mix, t2y));
+  if (sol_m) Fy += mad_rn(M.c, C.wall1, C.wall0);
+  if (sol_p) Fy -= mad_rn(M.c, C.wall1, C.wall0);
 }
 
 // The 9 staged populations of one node, population i at p[i * stride].
@@ -481,30 +543,46 @@ struct OffsetOut {
   }
 };
 
-// BGK toward f^eq(rho, u_eq) (Eqs. 2-3) plus the exact-difference term (Eq. 5),
-// written pairwise over opposite directions i, i': with cu = c_i.u, cd = c_i.du and
-// cs = c_i.(2u + du), omega f^eq_i + F_i = w_i (K + 4.5 rho (omega cu^2 + cd cs))
-// + 3 w_i rho (omega cu + cd), K = omega (drho - 1.5 rho u.u) - 1.5 rho du.(2u + du);
-// the direction i' flips the sign of the second term only.  fs(i): the pulled
-// population i of the node; fo(i): population i of the node in the output buffer.
+// BGK toward f^eq(rho, u) (Eqs. 2-3) plus the exact-difference term (Eq. 5),
+// f_i - omega (f_i - f^eq_i(u)) + f^eq_i(u + du) - f^eq_i(u)
+//   = keep (f_i - f^eq_i(u)) + f^eq_i(u + du),  keep = 1 - omega,
+// from the momentum j = rho u and the force F = rho du: with P = j + F and V = u + du the
+// quadratic parts XX = P_x V_x - keep j_x u_x, YY, XY and the linear part M = omega j + F give
+// every direction w_i (K + 4.5 (c_i c_i : quadratic)) + 3 w_i c_i.M, K = omega drho - 1.5 (XX + YY),
+// pairwise over opposite directions.  At tau_f = 1 keep is zero: nothing is left of f^eq(u) and of
+// the pulled populations.  fs(i): the pulled population i of the node; fo(i): population i of
+// the node in the output buffer.
 template <typename Real, typename Pops, typename Out>
-__device__ __forceinline__ void collide_f(const Pops& fs, const Out& fo, Real rho,
-                                          Real drho, Real ux, Real uy, Real dux, Real duy, Real omega_f) {
-  const Real sx = Real(2) * ux + dux, sy = Real(2) * uy + duy;
-  const Real usq = ux * ux + uy * uy;
-  const Real K = omega_f * (drho - Real(1.5) * rho * usq) - Real(1.5) * rho * (dux * sx + duy * sy);
-  const Real r45 = Real(4.5) * rho, r3 = Real(3) * rho, keep = Real(1) - omega_f;
-  auto pair = [&](int i, int j, Real cu, Real cd, Real cs, Real w) {
-    const Real sym = w * (K + r45 * (omega_f * cu * cu + cd * cs));
-    const Real anti = w * r3 * (omega_f * cu + cd);
-    fo(i) = keep * fs(i) + sym + anti;
-    fo(j) = keep * fs(j) + sym - anti;
+__device__ __forceinline__ void collide_f(const Pops& fs, const Out& fo, Real drho, Real jx, Real jy, Real Fx, Real Fy,
+                                          Real inv_rho, Real omega_f) {
+  const Real keep = Real(1) - omega_f;
+  const bool relax = omega_f != Real(1);
+  const Real w1 = lat_w<Real>(1), w5 = lat_w<Real>(5);
+  Real mx = jx + Fx, my = jy + Fy, d = drho;
+  const Real vx = mul_rn(mx, inv_rho), vy = mul_rn(my, inv_rho);
+  Real xx = mul_rn(mx, vx), yy = mul_rn(my, vy), xy = mul_rn(mx, vy);
+  if (relax) {
+    const Real kx = mul_rn(-keep, jx), ky = mul_rn(-keep, jy), ux = mul_rn(jx, inv_rho), uy = mul_rn(jy, inv_rho);
+    xx = mad_rn(kx, ux, xx);
+    yy = mad_rn(ky, uy, yy);
+    xy = mad_rn(kx, uy, xy);
+    mx = mad_rn(omega_f, jx, Fx);
+    my = mad_rn(omega_f, jy, Fy);
+    d = mul_rn(omega_f, drho);
+  }
+  const Real s = xx + yy;
+  const Real K = mad_rn(Real(-1.5), s, d);
+  const Real K1 = mul_rn(w1, K), K5 = mad_rn(Real(0.125), s, mul_rn(w5, K));
+  auto put = [&](int i, Real v) { fo(i) = relax ? mad_rn(keep, fs(i), v) : v; };
+  auto pair = [&](int i, int j, Real sym, Real w3, Real m) {
+    put(i, mad_rn(w3, m, sym));
+    put(j, mad_rn(-w3, m, sym));
   };
-  fo(0) = keep * fs(0) + lat_w<Real>(0) * K;
-  pair(1, 3, ux, dux, sx, lat_w<Real>(1));
-  pair(2, 4, uy, duy, sy, lat_w<Real>(2));
-  pair(5, 7, ux + uy, dux + duy, sx + sy, lat_w<Real>(5));
-  pair(6, 8, uy - ux, duy - dux, sy - sx, lat_w<Real>(6));
+  put(0, mul_rn(lat_w<Real>(0), K));
+  pair(1, 3, mad_rn(Real(0.5), xx, K1), Real(3) * w1, mx);
+  pair(2, 4, mad_rn(Real(0.5), yy, K1), Real(3) * w1, my);
+  pair(5, 7, mad_rn(Real(0.25), xy, K5), Real(3) * w5, mx + my);
+  pair(6, 8, mad_rn(Real(-0.25), xy, K5), Real(3) * w5, my - mx);
 }
 
 // Eq. 16 with g^eq of Eq. 18 and the source phi (second Eq. 19), pairwise as for f:
@@ -746,8 +824,9 @@ __device__ __forceinline__ void wall_temperature(Real (&gc)[9], bool lo, bool hi
 }
 
 // Shared memory (smem, interior_smem_bytes): per-thread rings of the staged f (FI_SLOTS rows)
-// and g (GI_SLOTS rows), then three-row rings of psi, u_act,x and u_act,y.  Each row's pull is
-// issued LOOKAHEAD iterations before it is used.
+// and g (GI_SLOTS rows), one row of psi (a node keeps what the force needs of the two rows
+// below in registers), then three-row rings of u_act,x and u_act,y.  Each row's pull is issued
+// LOOKAHEAD iterations before it is used.
 template <typename Real, bool THERMAL, int B>
 __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>& C, Real rra, const Tile& tile,
                                               long long step, bool local, unsigned char* smem, Real& acc_m,
@@ -756,8 +835,8 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
   constexpr int NS = B - 4;
   Real* const sF = reinterpret_cast<Real*>(smem);           // [FI_SLOTS][9][NS]
   Real* const sG = sF + FI_SLOTS * 9 * NS;                   // [GI_SLOTS][9][NS]
-  Real* const sPsi = sG + (THERMAL ? GI_SLOTS * 9 * NS : 0);  // [3][NS]
-  Real* const sUx = sPsi + 3 * NS;                           // [3][NS]
+  Real* const sPsi = sG + (THERMAL ? GI_SLOTS * 9 * NS : 0);  // [NS]
+  Real* const sUx = sPsi + NS;                               // [3][NS]
   Real* const sUy = sUx + 3 * NS;                            // [3][NS]
   const int tid = threadIdx.x;
   const bool act = tid < NS;
@@ -817,10 +896,11 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
     cp_async_commit();
   };
 
-  Real rho_p = Real(1), drho_p = Real(0), ux_p = Real(0), uy_p = Real(0), T_p = C.T0, dT_p = Real(0), coef_p = Real(0);
+  Real drho_p = Real(0), jx_p = Real(0), jy_p = Real(0), T_p = C.T0, dT_p = Real(0), coef_p = Real(0);
   Real inv_rho_p = Real(1);
+  PsiLine<Real> psM{Real(0), Real(0), Real(0)}, psS = psM;  // psi of rows r-1 and r-2 at this column
   Real T_p2 = C.T0, dT_p2 = Real(0), coef_p2 = Real(0);
-  // ring slots of row r = y0 - 2 + k: f (k mod FI_SLOTS), g (k mod GI_SLOTS), psi and u_act (k mod 3)
+  // ring slots of row r = y0 - 2 + k: f (k mod FI_SLOTS), g (k mod GI_SLOTS), u_act (k mod 3)
   int f_cur = 0, g_cur = 0, p_cur = 0;
 #pragma unroll
   for (int a = 0; a < LOOKAHEAD; ++a) issue_row(a, a, a);
@@ -833,7 +913,7 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
     const int p_prev = p_cur == 0 ? 2 : p_cur - 1;                 // row r-1
     const int p_prev2 = p_cur == 2 ? 0 : p_cur + 1;                // row r-2 (= r+1 = r-3)
     NodeState<Real> ns;
-    ns.rho = Real(1); ns.inv_rho = Real(1); ns.drho = Real(0); ns.ux = Real(0); ns.uy = Real(0);
+    ns.rho = Real(1); ns.inv_rho = Real(1); ns.drho = Real(0); ns.jx = Real(0); ns.jy = Real(0);
     ns.T = C.T0; ns.dT = Real(0); ns.coef = Real(0); ns.dpsi = Real(0);
     issue_row(k + LOOKAHEAD, f_issue, g_issue);
     cp_async_wait_lookahead<LOOKAHEAD>();  // this thread's copies of row r have landed
@@ -855,7 +935,7 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
       }
       ns = node_state<Real, THERMAL>(fc, gc, C, multiphase, false);
       bad_any = bad_any || ns.bad;
-      sPsi[p_cur * NS + s] = ns.dpsi;
+      sPsi[s] = ns.dpsi;
       if (out_col && r >= y0 && r < y1) {
         acc_m += ns.drho;
         if (THERMAL) {
@@ -868,34 +948,23 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
 
     // ===================== phase B: row q = r - 1 =====================
     const int q = r - 1;
-    if (f_col && q >= y0 - 1 && q >= 0 && q < ny) {
-      Real Fx = Real(0), Fy = Real(0);
-      if (multiphase) {
-        const Real* P0 = sPsi + p_prev * NS + s;
-        const Real* Pp = sPsi + p_cur * NS + s;
-        const Real* Pm = sPsi + p_prev2 * NS + s;
-        auto force = [&](Real dN, Real dNE, Real dNW, Real dS, Real dSE, Real dSW, bool sol_m, bool sol_p) {
-          sc_force<Real>(P0[0], P0[1], P0[-1], dN, dNE, dNW, dS, dSE, dSW, sol_m, sol_p, C, Fx, Fy);
-        };
-        if (q > 0 && q < ny - 1) {
-          force(Pp[0], Pp[1], Pp[-1], Pm[0], Pm[1], Pm[-1], false, false);
-        } else {
-          const bool sol_m = q == 0, sol_p = q == ny - 1;  // row q-1 / q+1 is a wall
-          force(sol_p ? Real(0) : Pp[0], sol_p ? Real(0) : Pp[1], sol_p ? Real(0) : Pp[-1], sol_m ? Real(0) : Pm[0],
-                sol_m ? Real(0) : Pm[1], sol_m ? Real(0) : Pm[-1], sol_m, sol_p);
+    PsiLine<Real> psN{Real(0), Real(0), Real(0)};  // zero beside a wall
+    if (f_col) {
+      if (multiphase && r >= 0 && r < ny) psN = psi_line<Real>(ns.dpsi, sPsi[s + 1], sPsi[s - 1]);
+      if (q >= y0 - 1 && q >= 0 && q < ny) {
+        Real Fx = Real(0), Fy = Real(0);
+        if (multiphase) sc_force<Real>(psN, psM, psS, q == 0, q == ny - 1, C, Fx, Fy);
+        Fy = mad_rn(drho_p + rra, -C.g_a, Fy);  // Eq. 14, gravity along -y
+        sUx[p_prev * NS + s] = mul_rn(mad_rn(Real(0.5), Fx, jx_p), inv_rho_p);  // Eq. 7
+        sUy[p_prev * NS + s] = mul_rn(mad_rn(Real(0.5), Fy, jy_p), inv_rho_p);
+        if (out_col && q >= y0 && q < y1) {
+          collide_f<Real>(StridedPops<Real>{sF + f_prev * 9 * NS + s, NS}, OffsetOut<Real>{Fout, q * pitch + xn, I},
+                          drho_p, jx_p, jy_p, Fx, Fy, inv_rho_p, C.omega_f);
         }
       }
-      Fy -= (drho_p + rra) * C.g_a;  // Eq. 14, gravity along -y
-      const Real inv_rho = sizeof(Real) == 8 ? inv_rho_p : fast_rcp(rho_p);
-      const Real dux = Fx * inv_rho, duy = Fy * inv_rho;
-      const Real uax = ux_p + Real(0.5) * dux, uay = uy_p + Real(0.5) * duy;  // Eq. 7
-      sUx[p_prev * NS + s] = uax;
-      sUy[p_prev * NS + s] = uay;
-      if (out_col && q >= y0 && q < y1) {
-        collide_f<Real>(StridedPops<Real>{sF + f_prev * 9 * NS + s, NS}, OffsetOut<Real>{Fout, q * pitch + xn, I},
-                          rho_p, drho_p, ux_p, uy_p, dux, duy, C.omega_f);
-      }
     }
+    psS = psM;
+    psM = psN;
     __syncthreads();
 
     // ===================== phase C: row q2 = r - 2 =====================
@@ -923,11 +992,10 @@ __device__ __forceinline__ void interior_rows(const Inst& I, const KConst<Real>&
     T_p2 = T_p;
     dT_p2 = dT_p;
     coef_p2 = coef_p;
-    rho_p = ns.rho;
     inv_rho_p = ns.inv_rho;
     drho_p = ns.drho;
-    ux_p = ns.ux;
-    uy_p = ns.uy;
+    jx_p = ns.jx;
+    jy_p = ns.jy;
     T_p = ns.T;
     dT_p = ns.dT;
     coef_p = ns.coef;
@@ -1007,8 +1075,8 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
   constexpr int NS = B - 4;
   Real* const sF = reinterpret_cast<Real*>(dyn_smem);               // [F_SLOTS][9][NS]
   Real* const sG = sF + F_SLOTS * 9 * NS;                           // [G_SLOTS][9][NS]
-  Real* const sPsi = sG + (THERMAL ? G_SLOTS * 9 * NS : 0);         // [3][NS]
-  Real* const sUx = sPsi + 3 * NS;                                  // [3][NS]
+  Real* const sPsi = sG + (THERMAL ? G_SLOTS * 9 * NS : 0);         // [NS]
+  Real* const sUx = sPsi + NS;                                      // [3][NS]
   Real* const sUy = sUx + 3 * NS;                                   // [3][NS]
   Real& sRra = sh.sRra;
   double (*sRed)[NPART] = sh.sRed;
@@ -1099,12 +1167,13 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
   double acc_open = 0.0;  // mass through the open ends (post_open)
   const bool zone_col = xn >= I.heater_x0 - I.heater_len && xn < I.heater_x0 + 2 * I.heater_len;
   // node scalars carried between iterations: row r-1 (f collision), row r-2 (g collision)
-  Real rho_p = Real(1), drho_p = Real(0), ux_p = Real(0), uy_p = Real(0), T_p = T0, dT_p = Real(0), coef_p = Real(0);
+  Real rho_p = Real(1), drho_p = Real(0), jx_p = Real(0), jy_p = Real(0), T_p = T0, dT_p = Real(0), coef_p = Real(0);
   Real inv_rho_p = Real(1);
+  PsiLine<Real> psM{Real(0), Real(0), Real(0)}, psS = psM;  // psi of rows r-1 and r-2 at this column
   Real T_p2 = T0, dT_p2 = Real(0), coef_p2 = Real(0);
   Real hm_p = Real(0), hm_p2 = Real(0);  // Hazi-Markus source term of rows r-1 and r-2
 
-  // ring slots: f and psi/u rings have 3 slots (row index mod 3), g has 4 (mod 4)
+  // ring slots: f and u rings have 3 slots (row index mod 3), g has 4 (mod 4)
   int f_cur = kbeg % F_SLOTS, g_cur = kbeg % G_SLOTS;
   issue_row(kbeg, f_cur, g_cur);
   for (int k = kbeg; k < kend; ++k) {
@@ -1121,7 +1190,7 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
     const bool row_ok = pery || (r >= 0 && r < ny);
     const int rn = pery ? wrap_index(r, ny) : r;
     NodeState<Real> ns;
-    ns.rho = Real(1); ns.inv_rho = Real(1); ns.drho = Real(0); ns.ux = Real(0); ns.uy = Real(0);
+    ns.rho = Real(1); ns.inv_rho = Real(1); ns.drho = Real(0); ns.jx = Real(0); ns.jy = Real(0);
     ns.T = T0; ns.dT = Real(0); ns.coef = Real(0); ns.dpsi = Real(0);
     if (col_ok && row_ok) {
       Real* fs = sF + f_cur * 9 * NS + s;
@@ -1143,7 +1212,7 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
       }
       ns = node_state<Real, THERMAL>(fc, gc, sC, multiphase, hazi);
       if (ns.bad) atomicOr(&st->status, STATUS_UNSTABLE);
-      sPsi[f_cur * NS + s] = ns.dpsi;
+      sPsi[s] = ns.dpsi;
       const bool out_row = r >= tile.y0 && r < tile.y1;
       if (post_open && !local && (inl || outl) && out_col && out_row) {
         // mass this node's pull took in minus the mass the pull let out of the lattice: in, the
@@ -1191,8 +1260,9 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
           }
         }
         if (MODE == MODE_STEP && channel && rn == ny / 2 && (xn == 1 || xn == nx - 2)) {
-          if (xn == 1) st->p_probe[2 * (step & 1)] = (double)ns.p;
-          if (xn == nx - 2) st->p_probe[2 * (step & 1) + 1] = (double)ns.p;
+          const double p = node_pressure<Real>(ns, sC, multiphase);
+          if (xn == 1) st->p_probe[2 * (step & 1)] = p;
+          if (xn == nx - 2) st->p_probe[2 * (step & 1) + 1] = p;
           __threadfence();
         }
       }
@@ -1217,33 +1287,25 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
     const int q = r - 1;
     // STEP needs u_act from row y0 - 1 (divergence at y0); FIELDS only on its output rows
     const int qmin = (MODE == MODE_STEP) ? tile.y0 - 1 : tile.y0;
+    PsiLine<Real> psN{Real(0), Real(0), Real(0)};  // zero beside a wall
+    if (multiphase && f_col && row_ok) psN = psi_line<Real>(ns.dpsi, sPsi[sp], sPsi[sm]);
     if (q >= qmin && f_col && (pery || (q >= 0 && q < ny))) {
-      const bool sol_m = !pery && q == 0;                // row q-1 is the bottom wall
-      const bool sol_p = !pery && !pool && q == ny - 1;  // row q+1 is the top wall
       Real Fx = Real(0), Fy = Real(0);
-      if (multiphase) {
-        const Real* P0 = sPsi + f_prev * NS;
-        // above the pool's top row: the zero-gradient ghost row repeats row q
-        const Real* Pp = (pool && q == ny - 1) ? P0 : sPsi + f_cur * NS;
-        const Real* Pm = sPsi + f_prev2 * NS;
-        sc_force<Real>(P0[s], P0[sp], P0[sm], sol_p ? Real(0) : Pp[s], sol_p ? Real(0) : Pp[sp],
-                       sol_p ? Real(0) : Pp[sm], sol_m ? Real(0) : Pm[s], sol_m ? Real(0) : Pm[sp],
-                       sol_m ? Real(0) : Pm[sm], sol_m, sol_p, sC, Fx, Fy);
-      }
-      Fy -= (drho_p + sRra) * sC.g_a;  // Eq. 14, gravity along -y
-      // FP64 reuses phase A's reciprocal (several FP64 instructions); FP32
-      // recomputes its cheap approximate one rather than hold another register
-      const Real inv_rho = sizeof(Real) == 8 ? inv_rho_p : fast_rcp(rho_p);
-      const Real dux = Fx * inv_rho, duy = Fy * inv_rho;
-      const Real uax = ux_p + Real(0.5) * dux, uay = uy_p + Real(0.5) * duy;  // Eq. 7
+      // above the pool's top row: the zero-gradient ghost row repeats row q
+      if (multiphase)
+        sc_force<Real>((pool && q == ny - 1) ? psM : psN, psM, psS, !pery && q == 0, !pery && !pool && q == ny - 1, sC,
+                       Fx, Fy);
+      Fy = mad_rn(drho_p + sRra, -sC.g_a, Fy);  // Eq. 14, gravity along -y
+      const Real uax = mul_rn(mad_rn(Real(0.5), Fx, jx_p), inv_rho_p);  // Eq. 7
+      const Real uay = mul_rn(mad_rn(Real(0.5), Fy, jy_p), inv_rho_p);
       sUx[f_prev * NS + s] = uax;
       sUy[f_prev * NS + s] = uay;
       const bool out_q = out_col && q >= tile.y0 && q < tile.y1;
       if (MODE == MODE_STEP && out_q) {
         collide_f<Real>(StridedPops<Real>{sF + f_prev * 9 * NS + s, NS}, plane_out(Fout, q * pitch + xn, plane, I.st, 9LL * plane),
-                        rho_p, drho_p, ux_p, uy_p, dux, duy, sC.omega_f);
-        if (channel && xn == 0) acc_fi += rho_p * uax;
-        if (channel && xn == nx - 1) acc_fo += rho_p * uax;
+                        drho_p, jx_p, jy_p, Fx, Fy, inv_rho_p, sC.omega_f);
+        if (channel && xn == 0) acc_fi += mad_rn(Real(0.5), Fx, jx_p);  // rho u_act
+        if (channel && xn == nx - 1) acc_fo += mad_rn(Real(0.5), Fx, jx_p);
       }
       if (MODE == MODE_FIELDS && out_q) {
         double* out = static_cast<double*>(I.f[(step + 1) & 1]);
@@ -1257,6 +1319,8 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
         }
       }
     }
+    psS = psM;
+    psM = psN;
     __syncthreads();
 
     // ===================== phase C: row q2 = r - 2 =====================
@@ -1293,8 +1357,8 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
     rho_p = ns.rho;
     inv_rho_p = ns.inv_rho;
     drho_p = ns.drho;
-    ux_p = ns.ux;
-    uy_p = ns.uy;
+    jx_p = ns.jx;
+    jy_p = ns.jy;
     T_p = ns.T;
     dT_p = ns.dT;
     coef_p = ns.coef;

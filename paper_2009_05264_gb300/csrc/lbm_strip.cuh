@@ -157,10 +157,10 @@ __device__ __forceinline__ void strip_rows(const Inst& I, const StripTile& t, fl
         float2 v[9];
         L.collide_f(o, drho_p, jx_p, jy_p, [&](int i) { return fB[i * 32]; }, v);
         L.store_row(t.fout, q, v);
-        if (EDGE && L.channel) {  // flux records
-          if (L.inl_a && L.out_a) S.fi += o.rho.x * uax.x;
-          if (L.outl_a && L.out_a) S.fo += o.rho.x * uax.x;
-          if (L.outl_b && L.out_b) S.fo += o.rho.y * uax.y;
+        if (EDGE && L.channel) {  // flux records, rho u_act = j + F / 2
+          if (L.inl_a && L.out_a) S.fi += __fmaf_rn(0.5f, o.Fx.x, jx_p.x);
+          if (L.outl_a && L.out_a) S.fo += __fmaf_rn(0.5f, o.Fx.x, jx_p.x);
+          if (L.outl_b && L.out_b) S.fo += __fmaf_rn(0.5f, o.Fx.y, jx_p.y);
         }
       }
     }

@@ -273,7 +273,7 @@ lbm_tma_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, u
   };
 
   float acc_m = 0.0f, acc_e = 0.0f, acc_h = 0.0f, acc_fi = 0.0f, acc_fo = 0.0f;
-  float rho_p = 1.0f, drho_p = 0.0f, ux_p = 0.0f, uy_p = 0.0f, T_p = T0, dT_p = 0.0f, coef_p = 0.0f;
+  float rho_p = 1.0f, drho_p = 0.0f, jx_p = 0.0f, jy_p = 0.0f, T_p = T0, dT_p = 0.0f, coef_p = 0.0f;
   float T_p2 = T0, dT_p2 = 0.0f, coef_p2 = 0.0f;
 
   // ring slots of row k: psi / u (mod 3), staged f (mod ST_FS) and g (mod ST_GS), with the
@@ -303,7 +303,7 @@ lbm_tma_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, u
     const bool row_ok = pery || (r >= 0 && r < ny);
     const int rn = pery ? wrap_index(r, ny) : r;
     NodeState<float> ns;
-    ns.rho = 1.0f; ns.drho = 0.0f; ns.ux = 0.0f; ns.uy = 0.0f;
+    ns.rho = 1.0f; ns.inv_rho = 1.0f; ns.drho = 0.0f; ns.jx = 0.0f; ns.jy = 0.0f;
     ns.T = T0; ns.dT = 0.0f; ns.coef = 0.0f; ns.dpsi = 0.0f;
     if (col_ok && row_ok) {
       float* const fs = sF + f_cur * ST_RW + (s + 2);
@@ -339,8 +339,9 @@ lbm_tma_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, u
           if (!pery && rn == 0 && xn >= I.heater_x0 && xn < I.heater_x0 + I.heater_len) acc_h += ns.dT;
         }
         if (channel && rn == ny / 2 && (xn == 1 || xn == nx - 2)) {
-          if (xn == 1) st->p_probe[2 * (step & 1)] = (double)ns.p;
-          if (xn == nx - 2) st->p_probe[2 * (step & 1) + 1] = (double)ns.p;
+          const double p = node_pressure<float>(ns, C, multiphase);
+          if (xn == 1) st->p_probe[2 * (step & 1)] = p;
+          if (xn == nx - 2) st->p_probe[2 * (step & 1) + 1] = p;
           __threadfence();
         }
       }
@@ -358,20 +359,20 @@ lbm_tma_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, u
         const float* P0 = sPsi + p_prev * NS;
         const float* Pp = sPsi + p_cur * NS;
         const float* Pm = sPsi + p_prev2 * NS;
-        sc_force<float>(P0[s], P0[sp], P0[sm], sol_p ? 0.0f : Pp[s], sol_p ? 0.0f : Pp[sp], sol_p ? 0.0f : Pp[sm],
-                        sol_m ? 0.0f : Pm[s], sol_m ? 0.0f : Pm[sp], sol_m ? 0.0f : Pm[sm], sol_m, sol_p, C, Fx, Fy);
+        const PsiLine<float> zero{0.0f, 0.0f, 0.0f};
+        sc_force<float>(sol_p ? zero : psi_line<float>(Pp[s], Pp[sp], Pp[sm]), psi_line<float>(P0[s], P0[sp], P0[sm]),
+                        sol_m ? zero : psi_line<float>(Pm[s], Pm[sp], Pm[sm]), sol_m, sol_p, C, Fx, Fy);
       }
-      Fy -= (drho_p + sRra) * C.g_a;  // Eq. 14, gravity along -y
+      Fy = mad_rn(drho_p + sRra, -C.g_a, Fy);  // Eq. 14, gravity along -y
       const float inv_rho = fast_rcp(rho_p);
-      const float dux = Fx * inv_rho, duy = Fy * inv_rho;
-      const float uax = ux_p + 0.5f * dux, uay = uy_p + 0.5f * duy;  // Eq. 7
+      const float uax = mul_rn(mad_rn(0.5f, Fx, jx_p), inv_rho), uay = mul_rn(mad_rn(0.5f, Fy, jy_p), inv_rho);  // Eq. 7
       sUx[p_prev * NS + s] = uax;
       sUy[p_prev * NS + s] = uay;
       if (out_col && q >= tile.y0 && q < tile.y1) {
         collide_f<float>(ShiftedPops{sF + f_prev * ST_RW + (s + 2)}, plane_out(Fout, q * pitch + xn, plane, I.st, 9LL * plane),
-                         rho_p, drho_p, ux_p, uy_p, dux, duy, C.omega_f);
-        if (channel && xn == 0) acc_fi += rho_p * uax;
-        if (channel && xn == nx - 1) acc_fo += rho_p * uax;
+                         drho_p, jx_p, jy_p, Fx, Fy, inv_rho, C.omega_f);
+        if (channel && xn == 0) acc_fi += mad_rn(0.5f, Fx, jx_p);
+        if (channel && xn == nx - 1) acc_fo += mad_rn(0.5f, Fx, jx_p);
       }
     }
     __syncthreads();
@@ -400,8 +401,8 @@ lbm_tma_kernel(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, u
     coef_p2 = coef_p;
     rho_p = ns.rho;
     drho_p = ns.drho;
-    ux_p = ns.ux;
-    uy_p = ns.uy;
+    jx_p = ns.jx;
+    jy_p = ns.jy;
     T_p = ns.T;
     dT_p = ns.dT;
     coef_p = ns.coef;
