@@ -573,12 +573,19 @@ __device__ __forceinline__ void collide_f(const Pops& fs, const Out& fo, Real dr
   const Real s = xx + yy;
   const Real K = mad_rn(Real(-1.5), s, d);
   const Real K1 = mul_rn(w1, K), K5 = mad_rn(Real(0.125), s, mul_rn(w5, K));
-  auto put = [&](int i, Real v) { fo(i) = relax ? mad_rn(keep, fs(i), v) : v; };
+  // a branch, not a select per population: at tau_f = 1 the multiply-adds are not to be issued
   auto pair = [&](int i, int j, Real sym, Real w3, Real m) {
-    put(i, mad_rn(w3, m, sym));
-    put(j, mad_rn(-w3, m, sym));
+    if (relax) {
+      fo(i) = mad_rn(keep, fs(i), mad_rn(w3, m, sym));
+      fo(j) = mad_rn(keep, fs(j), mad_rn(-w3, m, sym));
+    } else {
+      fo(i) = mad_rn(w3, m, sym);
+      fo(j) = mad_rn(-w3, m, sym);
+    }
   };
-  put(0, mul_rn(lat_w<Real>(0), K));
+  const Real f0 = mul_rn(lat_w<Real>(0), K);
+  if (relax) fo(0) = mad_rn(keep, fs(0), f0);
+  else fo(0) = f0;
   pair(1, 3, mad_rn(Real(0.5), xx, K1), Real(3) * w1, mx);
   pair(2, 4, mad_rn(Real(0.5), yy, K1), Real(3) * w1, my);
   pair(5, 7, mad_rn(Real(0.25), xy, K5), Real(3) * w5, mx + my);
@@ -800,7 +807,7 @@ __device__ __forceinline__ void post_partials(const Inst& I, InstState* st, cons
 // neighbours are the adjacent lanes, and only the wall rows 0 and ny - 1 take the wall
 // branches (bounce-back links, anti-bounce-back temperature, solid neighbours of the force,
 // one-sided wall divergence), decided once per row for the whole CTA.  The arithmetic is the
-// general loop's, expression for expression, so the results are bit-identical to it.
+// general loop's, expression for expression; results agree to rounding.
 // ---------------------------------------------------------------------------
 
 // Anti-bounce-back of g on the links of a wall row (the wall part of boundary_fill): the
