@@ -224,8 +224,10 @@ lbm_status lbm_load_state(lbm_ctx* ctx, const void* host_buf, size_t bytes);
  * cols - 8 columns, the other 8 cover halo columns; the one-column kernels run cols
  * threads, the FP32 strip kernel 1, 2 or 5 warps) and rows per CTA (>= 4, or the full height).
  * Results do not depend on the shape except through the per-CTA sums of the
- * domain-mean density (Eq. 14) and their rounding to the fixed-point totals; only speed differs.  0 = default: the band plan of
- * lbm_default_band_plan for the CTA slots of the current device and kernel form. */
+ * domain-mean density (Eq. 14) and their rounding to the fixed-point totals; only speed differs.
+ * rows 0 = default: the band plan of lbm_default_band_plan for the CTA slots of the current device
+ * and kernel form.  cols 0 = 128; with rows 0 too (and without this call) an FP64 lattice small
+ * enough that all its tiles are resident takes 64 columns and lower bands where that costs less. */
 lbm_status lbm_set_tiling(lbm_ctx* ctx, int32_t cols, int32_t rows);
 
 /* Time trial_steps steps of each candidate tiling (64, 128 and 256 columns, each with the

@@ -424,6 +424,7 @@ struct lbm_ctx {
   BandPlan plan{0, 0, 16};  // the step tiling's bands
   bool member = false;       // a batch steps it (and plans its own flat launch)
   bool rows_default = true;  // band height chosen by default_band_rows (re-chosen on changes)
+  bool cols_default = true;  // and the columns with it (fp64_tiling)
   int ntiles_step = 0, ntiles_aux = 0;
   int nopen_step = 0;  // step tiles with an open end (inlet or outlet columns)
   int flat_tiles = 0, flat_warps = 0, flat_grid = 0;  // the flat launch's tiles, warps per CTA and CTAs (0: none)
@@ -532,12 +533,49 @@ lbm_status plan_flat(lbm_ctx* c) {
 // asked for.
 bool use_flat(const lbm_ctx* c) { return c->flat_tiles > 0 && c->loop != LBM_LOOP_LAUNCHES; }
 
+// Tiling of an FP64 lattice whose default tiles (128 columns, bands of `rows`) are all resident:
+// 64 columns, with bands no higher, where that is cheaper.  The CTAs of an SM share its FP64 pipe,
+// and each CTA has its own chain of rows besides, so a step takes about
+//   (rows + 2) (cols ceil(tiles / SMs) + 98)
+// times 0.042 us: within 8 % of ten of the eleven tilings of 1000 x 100 measured (77 to 137 us a step).
+// default_band_plan counts CTA slots only: 1000 x 100 110.7 us a step with 128 columns and
+// bands of 5, 79.1 with 64 and 4; 256 x 256 103.4 and 61.7; 128 x 128 isothermal 38.9 and 36.1.
+bool fp64_small_rows(int nx, int ny, int sms, int& rows) {
+  auto tiles = [&](int cols, int r) {
+    return (long long)((nx + tile_cols(cols) - 1) / tile_cols(cols)) * ((ny + r - 1) / r);
+  };
+  auto cost = [&](int cols, int r) { return (r + 2.0) * (cols * (double)((tiles(cols, r) + sms - 1) / sms) + 98.0); };
+  double best = cost(128, rows);
+  bool better = false;
+  for (int r = rows; r >= std::min(kMinRows, ny); --r) {
+    if (tiles(64, r) > 4LL * sms || cost(64, r) >= best) continue;  // 4: the kernels' launch bounds
+    best = cost(64, r);
+    rows = r;
+    better = true;
+  }
+  return better;
+}
+
 // Re-choose the default tiling for the current kernel, precision and thermal flag.
 lbm_status retile_default(lbm_ctx* c, int cols) {
+  if (c->cols_default) cols = 128;
   const long long slots =
       step_wave_slots(c->prec == LBM_FP64, c->have_params ? c->thermal : 1, cols, step_kernel(c, cols),
                       step_flags(c->hinst));
-  const lbm_status s = set_tiling(c, cols, default_band_plan(c->nx, c->ny, cols, slots));
+  BandPlan plan = default_band_plan(c->nx, c->ny, cols, slots);
+  if (c->cols_default && c->prec == LBM_FP64 && plan.tall_count == 0) {
+    int dev = 0, sms = 0;
+    LBM_CUDA(c, cudaGetDevice(&dev));
+    LBM_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const long long tiles = (long long)((c->nx + tile_cols(128) - 1) / tile_cols(128)) *
+                            ((c->ny + plan.short_rows - 1) / plan.short_rows);
+    int rows = plan.short_rows;
+    if (tiles <= slots && fp64_small_rows(c->nx, c->ny, sms, rows)) {
+      cols = 64;
+      plan = BandPlan{0, 0, rows};
+    }
+  }
+  const lbm_status s = set_tiling(c, cols, plan);
   if (s != LBM_OK) return s;
   c->rows_default = true;
   return plan_flat(c);
@@ -1207,11 +1245,13 @@ lbm_status lbm_default_band_plan(int32_t nx, int32_t ny, int32_t cols, int64_t s
 
 lbm_status lbm_set_tiling(lbm_ctx* c, int32_t cols, int32_t rows) {
   if (!c) return LBM_EINVAL;
+  const bool cols_default = cols == 0 && rows == 0;
   if (cols == 0) cols = 128;
   if (!cols_supported(cols)) return fail(c, LBM_EINVAL, "cols must be 64, 128 or 256");
   if (rows < 0) return fail(c, LBM_EINVAL, "rows must be >= 0");
   DeviceGuard g(c->device);
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  c->cols_default = cols_default;
   if (rows == 0) return retile_default(c, cols);
   rows = std::min(rows, c->ny);
   if (rows < kMinRows && rows < c->ny) return fail(c, LBM_EINVAL, "rows must be >= 4 (or the full height)");
