@@ -368,12 +368,14 @@ def run_serve(n_requests: int, steps: int, rate: float = 2.0, seed: int = SEED +
 _CSRC = "paper_2009_05264_gb300/csrc/"
 # sources of each step-kernel form (scalar: also the FP64 step) and its ncu summary
 STEP_SOURCES = {"scalar": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h"),
-                "interior": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h"),
+                "interior": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h", _CSRC + "lbm_lane.cuh",
+                             _CSRC + "lbm_strip.cuh"),
                 "tma": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h", _CSRC + "lbm_tma.cuh")}
-PROFILES = {"interior": "profiles/lbm_fused_step_fp32_channel.md", "tma": "profiles/lbm_tma_step_fp32_channel.md"}
-KERNEL_LABELS = {"scalar": "lbm_fused_kernel (MODE_STEP)",
-                 "interior": "lbm_fused_kernel (MODE_STEP, interior path on tiles away from the open ends)",
-                 "paired": "lbm_pair_kernel (two columns per thread, packed FP32)",
+PROFILES = {"interior": "profiles/lbm_strip_step_fp32_channel.md", "tma": "profiles/lbm_tma_step_fp32_channel.md"}
+KERNEL_LABELS = {"fp64": "lbm_fused_kernel (MODE_STEP, interior path on tiles away from the open ends)",
+                 "scalar": "lbm_fused_kernel (MODE_STEP)",
+                 "interior": "lbm_strip_kernel (one warp per strip, two columns per lane, packed FP32)",
+                 "paired": "lbm_strip_kernel (one warp per strip, two columns per lane, packed FP32)",
                  "tma": "lbm_tma_kernel (MODE_STEP, rows staged by bulk tensor copies)"}
 
 
@@ -671,8 +673,8 @@ def run_ours(args):
                          "traffic_source": tsrc,
                          "peak_source": f"{peak_kind} HBM copy bandwidth",
                          "algorithmic_bytes_per_node": bpn,
-                         "kernel": KERNEL_LABELS[step_kernel] + (
-                             ", all timed steps in one lbm_persistent_kernel launch that overlaps consecutive steps"
+                         "kernel": KERNEL_LABELS["fp64" if prec == "fp64" and step_kernel == "interior" else step_kernel] + (
+                             ", all timed steps in one persistent launch that overlaps consecutive steps"
                              if loop == "overlapped" else "")},
             "e2e": {"value": e2e_value, "unit": "MLUPS",
                     "h2d_bytes_per_step": 4 * nodes * 8 / e2e_steps, "d2h_bytes_per_step": 4 * nodes * 8 / e2e_steps,
