@@ -78,7 +78,7 @@ bool build_flat_tiles(int inst, int nx, int ny, int geometry, int rows, std::vec
       FlatTile t{};
       t.inst = (short)inst;
       t.x0 = j * w;
-      t.wout = (short)w;
+      t.wout = (short)strip_columns(w, nx - t.x0);
       t.y0 = ystart(b);
       t.rows = ystart(b + 1) - t.y0;
       t.ntiles = ns * nb;

@@ -287,6 +287,10 @@ struct FlowPlan {
 // tiles for all the steps.  A tile of step s waits for the tiles around it (deps: what its pulls
 // read) to have finished step s - 1, and for the mass totals of step s - 1 to be complete.
 constexpr int FLAT_MAX_DEPS = 25;
+// Output columns of a strip of at most w (even) columns with `left` columns of the lattice from its
+// first on: what is left, rounded up to a lane's two.  The lanes past the last column of a lattice
+// that wraps then pull no column beyond those that the tile waits for.
+__host__ __device__ inline int strip_columns(int w, int left) { return left < w ? (left + 1) / 2 * 2 : w; }
 struct FlatTile {
   short inst, wout;            // output columns [x0, x0 + wout), rows [y0, y0 + rows)
   int x0, y0, rows;

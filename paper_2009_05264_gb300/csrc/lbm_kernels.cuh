@@ -1140,12 +1140,14 @@ __device__ __forceinline__ void fused_tile(const Inst* __restrict__ insts, const
   int xn = xc;
   bool col_ok = tid < NS;
   if (perx) {
+    // the last tile's columns past the halo would wrap to columns that an overlapped tile does not wait for
     xn = wrap_index(xc, nx);
+    col_ok = col_ok && xc < nx + 2;
   } else {
     col_ok = col_ok && xc >= 0 && xc < nx;
   }
   const bool out_col = tid >= 2 && tid < W + 2 && xc < nx;
-  const bool f_col = col_ok && s >= 1 && s <= W + 2;
+  const bool f_col = col_ok && s >= 1 && s <= W + 2 && xc <= nx;
   // shared-memory neighbours; at the open ends the ghost column repeats the end column
   const int sm = (!perx && xc == 0) ? s : s - 1;
   const int sp = (!perx && xc == nx - 1) ? s : s + 1;

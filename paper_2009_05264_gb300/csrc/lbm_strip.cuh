@@ -245,9 +245,9 @@ __device__ __forceinline__ void strip_tile(const Inst* __restrict__ insts, const
   strip_tile_consts<PCONST>(t, I, par, ts.step >= 0 ? ts.local : st->local_read != 0, post_open);
   t.y0 = uni(tile.y0);
   t.y1 = uni(tile.y1);
-  const int width = strip_width(cols);
-  t.wout = min(width, cols - 8 - w * width);
-  t.xs = uni(tile.x0) + w * width - 2;
+  const int width = strip_width(cols), x0 = uni(tile.x0) + w * width;
+  t.wout = strip_columns(min(width, cols - 8 - w * width), t.nx - x0);
+  t.xs = x0 - 2;
   float2* const ring = smem + w * 32 * 9 * strip_warp_slots(THERMAL, t.relax_f != 0);
   StripSums S{};
   if (t.xs + 2 < t.nx) {  // the last tile of a row may need fewer warps
