@@ -197,7 +197,7 @@ __device__ __forceinline__ bool flat_row(const Inst& I, const StripTile& t, cons
     if (L.hazi) L.history(rn, n);
     L.probes(rn, n, [&](int j, float p) { *reinterpret_cast<volatile double*>(&fs->slot[step & 3].probe[j]) = (double)p; });
   }
-  if (!ok) atomicOr(&st->status, STATUS_UNSTABLE);
+  if (L.bad(ok)) atomicOr(&st->status, STATUS_UNSTABLE);
   bar_sync(2, threads);
   if (*reinterpret_cast<volatile int*>(&sh.bad)) return false;
 

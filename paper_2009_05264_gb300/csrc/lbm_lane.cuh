@@ -93,7 +93,7 @@ struct LaneStep {
   bool perx, pery, channel, pool, multiphase, hazi, bubbles, local;
   int ca, cb;                     // columns of the two nodes (wrapped)
   unsigned oa, ob, om1, op1;      // byte offsets in a row: the nodes, and the columns beside them
-  bool in_a, in_b, inl_a, outl_a, outl_b, out_a, out_b;
+  bool inl_a, outl_a, outl_b, out_a, out_b;
 
   __device__ __forceinline__ LaneStep(const Inst& inst, const StripTile& tile)
       : I(inst), C(inst.strip.C), P(inst.strip.P), t(tile) {
@@ -115,7 +115,6 @@ struct LaneStep {
     int cm = xl - 1, cp = xl + 2;
     ca = xl;
     cb = xl + 1;
-    in_a = in_b = true;
     if (EDGE) {
       if (perx) {
         ca = wrap_index(xl, nx);
@@ -123,9 +122,7 @@ struct LaneStep {
         cm = wrap_index(xl - 1, nx);
         cp = wrap_index(xl + 2, nx);
       } else {
-        // columns outside the lattice read the end column: a valid state, never used
-        in_a = xl >= 0 && xl < nx;
-        in_b = xl + 1 >= 0 && xl + 1 < nx;
+        // columns outside the lattice read the end column: never used, and not checked (bad)
         ca = min(max(xl, 0), nx - 1);
         cb = min(max(xl + 1, 0), nx - 1);
         cm = min(max(xl - 1, 0), nx - 1);
@@ -254,14 +251,19 @@ struct LaneStep {
                 pg[i].x = __fmaf_rn(2.0f * lat_w<float>(i), C.dT_in, -pg[i].x);
           }
         }
-        if (outl_a) open_end(pf, 0, NodeBC{lo, hi, false, true, false});
+        if (outl_a) {
+          open_end(pf, 0, NodeBC{lo, hi, false, true, false});
+          // the lane's second column is outside: a copy, so that it is outside the EOS domain only with the node
+#pragma unroll
+          for (int i = 0; i < 9; ++i) pf[i].y = pf[i].x;
+        }
         if (outl_b) open_end(pf, 1, NodeBC{lo, hi, false, true, false});
         if (THERMAL && t.xs + t.wout + 3 >= nx - 1) {
           // zero temperature gradient: all nine populations of node nx - 2, wall links included
 #pragma unroll
           for (int i = 0; i < 9; ++i) {
             const float before = __shfl_up_sync(0xffffffffu, pg[i].y, 1);
-            if (outl_a) pg[i].x = before;
+            if (outl_a) pg[i].x = pg[i].y = before;
             if (outl_b) pg[i].y = pg[i].x;
           }
         }
@@ -392,6 +394,13 @@ struct LaneStep {
       n.coef = T;
       ok = ok && fabsf(T.x) < INFINITY && fabsf(T.y) < INFINITY;
     }
+  }
+
+  // Whether a node of the lattice was outside the EOS domain (ok: what node left of it over the lane's
+  // rows).  A lane with both columns beyond an open end holds none.
+  __device__ __forceinline__ bool bad(bool ok) const {
+    const int xl = t.xs + 2 * lane;
+    return !ok && !(EDGE && channel && (xl < 0 || xl >= nx));
   }
 
   // Hazi-Markus: the source's density-gradient term of this lane's output nodes of lattice row rn,

@@ -198,7 +198,7 @@ __device__ __forceinline__ void strip_rows(const Inst& I, const StripTile& t, fl
     psS = psM;
     psM = psN;
   }
-  S.bad = !ok;
+  S.bad = L.bad(ok);
   // sums of the output nodes only
   if (!L.out_a) S.m.x = S.e.x = 0.0f;
   if (!L.out_b) S.m.y = S.e.y = 0.0f;
