@@ -14,8 +14,8 @@ cudaError_t launch_flat(int thermal, int flags, int warps, const Inst* d_inst, c
   if (flat_resident_ctas(thermal, flags, h_inst != nullptr, warps) < 1) return cudaErrorInvalidConfiguration;
   const int insts = h_inst ? 0 : (ntiles + grid - 1) / grid;
   auto go = [&](auto fn) -> cudaError_t {
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)flat_smem_bytes(flags, warps, insts));
+    // the limit of every launch of this kernel: other threads' lattices share the attribute
+    const cudaError_t e = flat_set_smem_limit(fn);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

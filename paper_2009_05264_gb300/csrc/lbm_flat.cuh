@@ -482,10 +482,14 @@ lbm_flat_kernel(const Inst* __restrict__ insts, const FlatTile* __restrict__ til
 // Host launchers.
 // ---------------------------------------------------------------------------
 template <typename Kernel>
+cudaError_t flat_set_smem_limit(Kernel fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)flat_smem_bytes(STEP_RELAX, FLAT_MAX_WARPS, FLAT_MAX_ROUNDS));
+}
+template <typename Kernel>
 int flat_resident(Kernel fn, int flags, int warps, int insts) {
   int n = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)flat_smem_bytes(STEP_RELAX, FLAT_MAX_WARPS, FLAT_MAX_ROUNDS)) != cudaSuccess ||
+  if (flat_set_smem_limit(fn) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, 32 * warps, flat_smem_bytes(flags, warps, insts)) !=
           cudaSuccess)
     return 0;
