@@ -62,7 +62,8 @@ struct FlatShared {
   int local0[FLAT_MAX_ROUNDS];
   FlatRow row[2][FLAT_MAX_WARPS];
   double rho[2];
-  int bad;  // a wait gave up
+  // a wait of turn t gave up: word t & 1, which nobody writes again before all the turn's warps have read it
+  int bad[2];
   // completed steps for the finishing warp, by turns: the instance's position among the CTA's tiles
   // (-1: the launch is over) and the step's number
   int fin_round[2];
@@ -144,7 +145,7 @@ __device__ __forceinline__ bool flat_row(const Inst& I, const StripTile& t, cons
       if (L.lane < ft.ndeps)
         got = flat_wait(done + (size_t)ft.deps[L.lane] * FLAT_DONE_STRIDE, (unsigned)k * ft.dep_rows[L.lane], bar,
                         max_polls);
-      if (!__all_sync(0xffffffffu, got) && L.lane == 0) *reinterpret_cast<volatile int*>(&sh.bad) = 1;
+      if (!__all_sync(0xffffffffu, got) && L.lane == 0) *reinterpret_cast<volatile int*>(&sh.bad[turn & 1]) = 1;
     }
     bar_sync(5, threads - 32);
   }
@@ -199,7 +200,7 @@ __device__ __forceinline__ bool flat_row(const Inst& I, const StripTile& t, cons
   }
   if (L.bad(ok)) atomicOr(&st->status, STATUS_UNSTABLE);
   bar_sync(2, threads);
-  if (*reinterpret_cast<volatile int*>(&sh.bad)) return false;
+  if (*reinterpret_cast<volatile int*>(&sh.bad[turn & 1])) return false;
 
   // ===================== phase B: force, u_act, f collision =====================
   typename Step::Flow o;
@@ -282,12 +283,12 @@ __device__ __forceinline__ bool flat_serve(const Inst& I, const StripTile& t, co
     rho = ((double)m * I.fix_unscale[0] + nn * I.rho_ref) / nn;
   }
   if (lane == 0) {
-    if (!got) *reinterpret_cast<volatile int*>(&sh.bad) = 1;
+    if (!got) *reinterpret_cast<volatile int*>(&sh.bad[turn & 1]) = 1;
     sh.rho[turn & 1] = rho;
   }
   __syncwarp();
   bar_sync(2, threads);
-  if (*reinterpret_cast<volatile int*>(&sh.bad)) return false;
+  if (*reinterpret_cast<volatile int*>(&sh.bad[turn & 1])) return false;
 
   // the mass, which every tile of the next step waits for
   const bool pery = t.geometry == GEOM_PERIODIC, channel = t.geometry == GEOM_CHANNEL;
@@ -395,7 +396,7 @@ lbm_flat_kernel(const Inst* __restrict__ insts, const FlatTile* __restrict__ til
     reinterpret_cast<int*>(&sh.tile[rd])[w] =
         reinterpret_cast<const int*>(tiles + blockIdx.x + (size_t)rd * gridDim.x)[w];
   }
-  if (threadIdx.x == 0) sh.bad = 0;
+  if (threadIdx.x == 0) sh.bad[0] = sh.bad[1] = 0;
   __syncthreads();
   if ((int)threadIdx.x < rounds) {
     const int rd = threadIdx.x;
