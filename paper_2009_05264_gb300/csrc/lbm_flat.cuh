@@ -84,6 +84,11 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ long long ld_acquire(const long long* p) {
+  long long v;
+  asm volatile("ld.acquire.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ void red_release(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -273,10 +278,15 @@ __device__ __forceinline__ bool flat_serve(const Inst& I, const StripTile& t, co
   double rho = rho_first;
   bool got = true;
   if (k > 0) {
-    got = flat_wait(&fs->slot[slot_prev].count, (unsigned)ft.ntiles, bar, max_polls);
-    // this step's slot: its totals of four steps back have been taken and cleared
-    unsigned polls = 0;
-    if (got) got = flow_wait<long long>(&st->step, step - 2 < step - k ? step - k : step - 2, bar, max_polls, polls, global_ns());
+    // this step's slot: its totals of four steps back have been taken and cleared (first: the other
+    // wait is the longer one)
+    const long long cleared = step - 2 < step - k ? step - k : step - 2;
+    if (ld_acquire(&st->step) < cleared) {
+      unsigned polls = 0;
+      got = flow_wait<long long>(&st->step, cleared, bar, max_polls, polls, global_ns());
+      fence_gpu();  // the clears are seen before this tile adds
+    }
+    if (got) got = flat_wait(&fs->slot[slot_prev].count, (unsigned)ft.ntiles, bar, max_polls);
     // as finish_step forms it: the same totals give the same mean
     const double nn = (double)I.nx * (double)I.ny;
     const long long m = *reinterpret_cast<const volatile long long*>(&fs->slot[slot_prev].sums[0]);
@@ -370,14 +380,15 @@ __device__ __forceinline__ void flat_finish(const Inst& I, FlatState* fs, long l
   double tot[NPART];
 #pragma unroll
   for (int j = 0; j < NPART; ++j) tot[j] = __shfl_sync(0xffffffffu, x, j);
+  __threadfence();  // every lane's clears are performed before the step count, after which the slot is used again
+  __syncwarp();
   if (lane == 0) {
     fs->slot[slot_prev].count = 0u;
     fs->slot[slot_prev].complete = 0u;
     st->p_probe[2 * (step & 1)] = *reinterpret_cast<const volatile double*>(&fs->slot[slot].probe[0]);
     st->p_probe[2 * (step & 1) + 1] = *reinterpret_cast<const volatile double*>(&fs->slot[slot].probe[1]);
-    finish_step<THERMAL, MODE_STEP>(I, st, tot, step);
+    finish_step<THERMAL, MODE_STEP>(I, st, tot, step);  // fences before it publishes the step count
   }
-  __threadfence();
   __syncwarp();
 }
 
