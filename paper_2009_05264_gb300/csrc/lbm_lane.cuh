@@ -435,12 +435,10 @@ struct LaneStep {
       }
     }
   }
-  // Heater-row temperature of this lane's output nodes of row 0.
-  __device__ __forceinline__ float heater_dT(const float2& dT) const {
-    float h = 0.0f;
-    if (out_a && ca >= I.heater_x0 && ca < I.heater_x0 + I.heater_len) h += dT.x;
-    if (out_b && cb >= I.heater_x0 && cb < I.heater_x0 + I.heater_len) h += dT.y;
-    return h;
+  // Heater-row temperatures of this lane's output nodes of row 0 (zero beside the heater).
+  __device__ __forceinline__ float2 heater_dT(const float2& dT) const {
+    return make_float2(out_a && ca >= I.heater_x0 && ca < I.heater_x0 + I.heater_len ? dT.x : 0.0f,
+                       out_b && cb >= I.heater_x0 && cb < I.heater_x0 + I.heater_len ? dT.y : 0.0f);
   }
 
   // East and west neighbours of a row's values, from the adjacent lanes; at the open ends the
