@@ -627,7 +627,7 @@ lbm_status launch(lbm_ctx* c, int mode) {
 // Fill the device instance descriptor from validated parameters.
 lbm_status apply_params(lbm_ctx* c, const lbm_params* p) {
   if (const char* why = check_params(c->nx, c->ny, p)) return fail(c, LBM_EINVAL, why);
-  Inst& I = c->hinst;
+  Inst I;  // the context keeps its descriptor (a kernel parameter of its launches) when p is refused
   if (const char* why = fill_inst(I, p, c->nx, c->ny, c->L.pitch, c->L.plane, c->prec == LBM_FP64))
     return fail(c, LBM_EINVAL, why);
   for (int b = 0; b < 2; ++b) {
@@ -639,6 +639,7 @@ lbm_status apply_params(lbm_ctx* c, const lbm_params* p) {
   I.st = c->d_state;
   I.sums = reinterpret_cast<unsigned long long*>(c->base + c->L.off_sums);
   I.ring = reinterpret_cast<double*>(c->base + c->L.off_ring);
+  c->hinst = I;
   LBM_CUDA(c, cudaMemcpyAsync(c->d_inst, &c->hinst, sizeof(Inst), cudaMemcpyHostToDevice, c->stream));
   c->params = *p;
   c->thermal = p->thermal;
