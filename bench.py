@@ -259,7 +259,7 @@ def run_c2(steps: int = 2000, nx: int = 1000, ny: int = 100):
         lat.sync()
         ms = e0.elapsed_time(e1)
         out[prec] = {"value": nx * ny * n / (ms * 1e-3) / 1e6, "unit": "MLUPS", "steps": n, "ms_per_step": ms / n,
-                     "kernel": lat.step_kernel, "tiling": f"autotuned {tuned[0]}x{tuned[1] or 'default plan'}",
+                     "kernel": lat.step_form, "tiling": f"autotuned {tuned[0]}x{tuned[1] or 'default plan'}",
                      "autotune_s": tune_s}
         lat.close()
     return out
@@ -287,7 +287,7 @@ def run_batch(steps: int, trial_steps: int = 4, n: int = 64, seed: int = SEED + 
     cols, rows = b.autotune(trial_steps=trial_steps)
     tune_s = time.perf_counter() - t0
     b.step(3)
-    loop = b.step_loop
+    loop, form = b.step_loop, b.step_form
     st = b.stream
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     l0 = b.launches
@@ -316,7 +316,7 @@ def run_batch(steps: int, trial_steps: int = 4, n: int = 64, seed: int = SEED + 
             "nodes": nodes, "steps": steps, "value": batched, "unit": "MLUPS", "ms_per_step": ms_b / steps,
             "sequential": {"value": seq, "unit": "MLUPS", "ms_per_step": ms_s / steps,
                            "how": "each lattice alone through lbm_step_async, one after another"},
-            "speedup_vs_sequential": batched / seq, "tiling": f"{cols}x{rows}", "loop": loop, "autotune_s": tune_s,
+            "speedup_vs_sequential": batched / seq, "tiling": f"{cols}x{rows}", "loop": loop, "kernel": form, "autotune_s": tune_s,
             "gpu_launches": launches, "launches_sequential": n * steps, "finite": bool(ok),
             "members_finite": sum(member_ok), "members": len(member_ok),
             "solves_per_hour_50k_steps": n * 3600.0 / (50000 * ms_b * 1e-3 / steps),
@@ -366,16 +366,16 @@ def run_serve(n_requests: int, steps: int, rate: float = 2.0, seed: int = SEED +
 
 
 _CSRC = "paper_2009_05264_gb300/csrc/"
-# sources of each step-kernel form (scalar: also the FP64 step) and its ncu summary
+# sources of each step kernel (scalar: also the FP64 step with its interior path) and its ncu summary
 STEP_SOURCES = {"scalar": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h"),
-                "interior": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h", _CSRC + "lbm_lane.cuh",
-                             _CSRC + "lbm_strip.cuh"),
+                "strip": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h", _CSRC + "lbm_lane.cuh",
+                          _CSRC + "lbm_strip.cuh"),
                 "tma": (_CSRC + "lbm_kernels.cuh", _CSRC + "lbm_internal.h", _CSRC + "lbm_tma.cuh")}
-PROFILES = {"interior": "profiles/lbm_strip_step_fp32_channel.md", "tma": "profiles/lbm_tma_step_fp32_channel.md"}
-KERNEL_LABELS = {"fp64": "lbm_fused_kernel (MODE_STEP, interior path on tiles away from the open ends)",
+PROFILES = {"strip": "profiles/lbm_strip_step_fp32_channel.md", "tma": "profiles/lbm_tma_step_fp32_channel.md"}
+KERNEL_LABELS = {"interior": "lbm_fused_kernel (MODE_STEP, interior path on tiles away from the open ends)",
                  "scalar": "lbm_fused_kernel (MODE_STEP)",
-                 "interior": "lbm_strip_kernel (one warp per strip, two columns per lane, packed FP32)",
-                 "paired": "lbm_strip_kernel (one warp per strip, two columns per lane, packed FP32)",
+                 "strip": "lbm_strip_kernel (one warp per strip, two columns per lane, packed FP32)",
+                 "flat": "lbm_flat_kernel (one warp per row, two columns per lane, packed FP32)",
                  "tma": "lbm_tma_kernel (MODE_STEP, rows staged by bulk tensor copies)"}
 
 
@@ -590,7 +590,7 @@ def run_ours(args):
         lat.set_tiling(c, r)
     lat.set_kernel(args.kernel)
     lat.set_step_loop(args.loop)
-    step_kernel = lat.step_kernel  # the form the timed launches take
+    step_kernel = lat.step_form  # the kernel that the timed call runs
     t = lat.tiling
     tiling_desc = (f"{t['cols']} columns; per strip {t['tall_count']} bands of {t['tall_rows']} rows, then bands of "
                    f"{t['short_rows']}" + ("" if args.tiling else " (default plan)"))
@@ -673,7 +673,7 @@ def run_ours(args):
                          "traffic_source": tsrc,
                          "peak_source": f"{peak_kind} HBM copy bandwidth",
                          "algorithmic_bytes_per_node": bpn,
-                         "kernel": KERNEL_LABELS["fp64" if prec == "fp64" and step_kernel == "interior" else step_kernel] + (
+                         "kernel": KERNEL_LABELS[step_kernel] + (
                              ", all timed steps in one persistent launch that overlaps consecutive steps"
                              if loop == "overlapped" else "")},
             "e2e": {"value": e2e_value, "unit": "MLUPS",

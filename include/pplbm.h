@@ -280,9 +280,18 @@ enum { LBM_KERNEL_AUTO = 0, LBM_KERNEL_SCALAR = 1, LBM_KERNEL_PAIRED = 2, LBM_KE
 lbm_status lbm_set_kernel(lbm_ctx* ctx, int32_t kernel);
 /* The form (LBM_KERNEL_SCALAR, _INTERIOR, _PAIRED or _TMA) the context's step launches go by
  * with its current kernel request, precision, parameters and tiling (_SCALAR where the pool
- * geometry, the Hazi-Markus source or the bubble statistics need the per-node boundary logic,
- * whichever kernel runs it); -1 if ctx is NULL. */
+ * geometry, the Hazi-Markus source or the bubble statistics need the per-node boundary logic);
+ * -1 if ctx is NULL.  It names the request as resolved, not the kernel: lbm_step_form does. */
 int32_t lbm_step_kernel(const lbm_ctx* ctx);
+/* The kernel that a multi-step call runs now, with the context's kernel and loop requests,
+ * precision, parameters and tiling; -1 if ctx is NULL.
+ *   LBM_FORM_SCALAR: one column per thread, boundary logic per node (FP64, or as asked for).
+ *   LBM_FORM_INTERIOR: the same with a path without boundary logic for inner tiles (FP64).
+ *   LBM_FORM_TMA: one column per thread, rows staged by bulk tensor copies (FP32, as asked for).
+ *   LBM_FORM_STRIP: FP32, one warp per strip, two columns per lane.
+ *   LBM_FORM_FLAT: FP32, one CTA per tile and one warp per row, all steps in one launch. */
+enum { LBM_FORM_SCALAR = 1, LBM_FORM_INTERIOR = 2, LBM_FORM_TMA = 3, LBM_FORM_STRIP = 4, LBM_FORM_FLAT = 5 };
+int32_t lbm_step_form(const lbm_ctx* ctx);
 
 /* How lbm_step / lbm_step_async advance the lattice (a calling convention of the library;
  * the paper's time loop, Sec. 2 and Fig. 2, is the same either way).
@@ -390,6 +399,9 @@ lbm_status lbm_batch_set_step_loop(lbm_batch* b, int32_t loop);
 /* The loop a multi-step call takes now (LBM_LOOP_LAUNCHES, _PERSISTENT or _OVERLAPPED); -1 on
  * error. */
 int32_t lbm_batch_step_loop(lbm_batch* b);
+/* The kernel that a multi-step call of the batch runs now (LBM_FORM_*, as lbm_step_form); -1 if b is
+ * NULL or its tables cannot be built. */
+int32_t lbm_batch_step_form(lbm_batch* b);
 /* As lbm_set_wait_limit, for the batch's persistent and TMA launches. */
 lbm_status lbm_batch_set_wait_limit(lbm_batch* b, int64_t max_polls);
 /* lbm_read_fields of one member. */

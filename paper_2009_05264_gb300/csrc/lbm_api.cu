@@ -1154,6 +1154,11 @@ int32_t lbm_step_kernel(const lbm_ctx* c) {
                          c->params.source_model == LBM_SOURCE_HAZI_MARKUS);
 }
 
+int32_t lbm_step_form(const lbm_ctx* c) {
+  if (!c) return -1;
+  return executed_form(step_kernel(c, c->cols), use_flat(c));
+}
+
 lbm_status lbm_set_step_loop(lbm_ctx* c, int32_t loop) {
   if (!c) return LBM_EINVAL;
   if (loop < LBM_LOOP_AUTO || loop > LBM_LOOP_PERSISTENT)

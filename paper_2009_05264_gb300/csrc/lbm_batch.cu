@@ -521,6 +521,16 @@ int32_t lbm_batch_step_loop(lbm_batch* b) {
   return out;
 }
 
+int32_t lbm_batch_step_form(lbm_batch* b) {
+  if (!b) return -1;
+  int prev = -1;
+  cudaGetDevice(&prev);
+  cudaSetDevice(b->device);
+  const int32_t out = !b->dirty || rebuild(b) == LBM_OK ? executed_form(b->launch_kernel, batch_flat(b)) : -1;
+  if (prev >= 0) cudaSetDevice(prev);
+  return out;
+}
+
 lbm_status lbm_batch_set_wait_limit(lbm_batch* b, int64_t max_polls) {
   if (!b) return LBM_EINVAL;
   if (max_polls < 0 || max_polls > 0xffffffffll) return bfail(b, LBM_EINVAL, "max_polls out of range");

@@ -413,6 +413,12 @@ inline int reported_kernel(int requested, int form, bool full, bool hazi) {
   if (requested == LBM_KERNEL_PAIRED) return hazi ? LBM_KERNEL_SCALAR : LBM_KERNEL_PAIRED;
   return full ? LBM_KERNEL_SCALAR : LBM_KERNEL_INTERIOR;
 }
+// The LBM_FORM_* value of the kernel that runs.
+inline int executed_form(int form, bool flat) {
+  if (flat) return LBM_FORM_FLAT;
+  return form == FORM_STRIP ? LBM_FORM_STRIP : form == LBM_KERNEL_TMA ? LBM_FORM_TMA
+         : form == LBM_KERNEL_INTERIOR ? LBM_FORM_INTERIOR : LBM_FORM_SCALAR;
+}
 // Whether a kernel has a persistent form.
 inline bool has_persistent(int form) {
   return form == LBM_KERNEL_SCALAR || form == LBM_KERNEL_INTERIOR || form == FORM_STRIP;

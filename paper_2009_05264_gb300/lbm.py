@@ -32,12 +32,13 @@ EXPORTS = (
     "lbm_set_populations", "lbm_read_diagnostics", "lbm_read_diagnostics_range", "lbm_state_bytes",
     "lbm_save_state", "lbm_load_state",
     "lbm_set_tiling", "lbm_autotune", "lbm_get_tiling", "lbm_default_band_plan", "lbm_set_kernel", "lbm_step_kernel",
+    "lbm_step_form",
     "lbm_set_step_loop", "lbm_step_loop", "lbm_set_wait_limit", "lbm_get_step", "lbm_launch_count", "lbm_get_stream",
     "lbm_critical_temperature",
     "lbm_destroy", "lbm_status_string", "lbm_last_error", "lbm_step_noalloc", "lbm_probe_fma_rate",
     "lbm_batch_create", "lbm_batch_add", "lbm_batch_remove", "lbm_batch_member", "lbm_batch_size",
     "lbm_batch_set_tiling", "lbm_batch_set_kernel", "lbm_batch_get_tiling", "lbm_batch_autotune", "lbm_batch_step",
-    "lbm_batch_step_async", "lbm_batch_sync", "lbm_batch_set_step_loop", "lbm_batch_step_loop",
+    "lbm_batch_step_async", "lbm_batch_sync", "lbm_batch_set_step_loop", "lbm_batch_step_loop", "lbm_batch_step_form",
     "lbm_batch_set_wait_limit", "lbm_batch_read_fields", "lbm_batch_launch_count",
     "lbm_batch_get_stream", "lbm_batch_last_error", "lbm_batch_destroy",
 )
@@ -46,6 +47,7 @@ EXPORTS = (
 KERNELS = {"auto": 0, "scalar": 1, "paired": 2, "tma": 3, "interior": 4}
 KERNEL_NAMES = {v: k for k, v in KERNELS.items()}
 LOOPS = {"auto": 0, "launches": 1, "persistent": 2}
+FORM_NAMES = {1: "scalar", 2: "interior", 3: "tma", 4: "strip", 5: "flat"}
 LOOP_NAMES = {0: "auto", 1: "launches", 2: "persistent", 3: "overlapped"}
 
 
@@ -112,6 +114,7 @@ def load(build_if_missing: bool = True, path: str | None = None):
         "lbm_set_tiling": (ctypes.c_int, [vp, i32, i32]),
         "lbm_set_kernel": (ctypes.c_int, [vp, i32]),
         "lbm_step_kernel": (i32, [vp]),
+        "lbm_step_form": (i32, [vp]),
         "lbm_set_step_loop": (ctypes.c_int, [vp, i32]),
         "lbm_step_loop": (i32, [vp]),
         "lbm_set_wait_limit": (ctypes.c_int, [vp, i64]),
@@ -141,6 +144,7 @@ def load(build_if_missing: bool = True, path: str | None = None):
         "lbm_batch_step_async": (ctypes.c_int, [vp, i64]),
         "lbm_batch_set_step_loop": (ctypes.c_int, [vp, i32]),
         "lbm_batch_step_loop": (i32, [vp]),
+        "lbm_batch_step_form": (i32, [vp]),
         "lbm_batch_set_wait_limit": (ctypes.c_int, [vp, i64]),
         "lbm_batch_sync": (ctypes.c_int, [vp, ctypes.POINTER(i32)]),
         "lbm_batch_read_fields": (ctypes.c_int, [vp, i32, dp, dp, dp, dp, sz]),
@@ -265,8 +269,15 @@ class Lattice:
 
     @property
     def step_kernel(self) -> str:
-        """The kernel form the step launches take ("scalar", "interior", "paired" or "tma")."""
+        """The form asked for, as resolved ("scalar", "interior", "paired" or "tma"); `step_form` names
+        the kernel that runs."""
         return KERNEL_NAMES[int(self._L.lbm_step_kernel(self._h))]
+
+    @property
+    def step_form(self) -> str:
+        """The kernel that a multi-step call runs now: "scalar" or "interior" (one column per thread),
+        "tma", "strip" (a warp per strip of columns) or "flat" (a CTA per tile, a warp per row)."""
+        return FORM_NAMES[int(self._L.lbm_step_form(self._h))]
 
     def set_step_loop(self, loop: str):
         """How multi-step calls run: "auto", "launches" (one launch per step) or "persistent"
@@ -465,6 +476,11 @@ class Batch:
     @property
     def step_loop(self) -> str:
         return LOOP_NAMES[int(self._L.lbm_batch_step_loop(self._h))]
+
+    @property
+    def step_form(self) -> str:
+        """The kernel that a multi-step call of the batch runs now (as Lattice.step_form)."""
+        return FORM_NAMES[int(self._L.lbm_batch_step_form(self._h))]
 
     def set_wait_limit(self, max_polls: int):
         self._check(self._L.lbm_batch_set_wait_limit(self._h, int(max_polls)))
