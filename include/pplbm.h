@@ -230,10 +230,11 @@ lbm_status lbm_load_state(lbm_ctx* ctx, const void* host_buf, size_t bytes);
  * enough that all its tiles are resident takes 64 columns and lower bands where that costs less. */
 lbm_status lbm_set_tiling(lbm_ctx* ctx, int32_t cols, int32_t rows);
 
-/* Time trial_steps steps of each candidate tiling (64, 128 and 256 columns, each with the
- * default plan and with uniform bands of 4, 7, 10, 16, 24, 32 and 48 rows where the lattice
- * is that high) and keep the fastest; the chosen columns and rows (0 = default plan) go to
- * *cols and *rows (either may be NULL).  The trials advance the lattice: re-initialise it
+/* Time trial_steps steps of each candidate tiling (the default tiling of lbm_set_tiling(0, 0); 64,
+ * 128 and 256 columns, each with the default plan and with uniform bands of 4, 7, 10, 16, 24, 32
+ * and 48 rows where the lattice is that high) and keep the fastest; the chosen columns and rows
+ * (0 = default plan) go to *cols and *rows (either may be NULL; lbm_set_tiling with them gives the
+ * same tiling).  The trials advance the lattice: re-initialise it
  * afterwards if its state matters.  Results depend on the tiling only through the per-CTA
  * sums of the domain-mean density.  Errors: LBM_EINVAL (trial_steps < 1), LBM_ESTATE (no
  * parameters), LBM_EUNSTABLE, LBM_ECUDA. */

@@ -424,7 +424,7 @@ struct lbm_ctx {
   BandPlan plan{0, 0, 16};  // the step tiling's bands
   bool member = false;       // a batch steps it (and plans its own flat launch)
   bool rows_default = true;  // band height chosen by default_band_rows (re-chosen on changes)
-  bool cols_default = true;  // and the columns with it (fp64_tiling)
+  bool cols_default = true;  // and the columns with it (fp64_small_rows)
   int ntiles_step = 0, ntiles_aux = 0;
   int nopen_step = 0;  // step tiles with an open end (inlet or outlet columns)
   int flat_tiles = 0, flat_warps = 0, flat_grid = 0;  // the flat launch's tiles, warps per CTA and CTAs (0: none)
@@ -540,6 +540,10 @@ bool use_flat(const lbm_ctx* c) { return c->flat_tiles > 0 && c->loop != LBM_LOO
 // times 0.042 us: within 8 % of ten of the eleven tilings of 1000 x 100 measured (77 to 137 us a step).
 // default_band_plan counts CTA slots only: 1000 x 100 110.7 us a step with 128 columns and
 // bands of 5, 79.1 with 64 and 4; 256 x 256 103.4 and 61.7; 128 x 128 isothermal 38.9 and 36.1.
+// The constants are those of a thermal step.  Checked on fourteen other lattices (walls, 128 x 128 to
+// 1500 x 60) against 64 and 128 columns with bands of 4 to 10: the chosen tiling is within 2.5 % of
+// the best of the twelve on all eleven thermal ones (300 x 257 69.9 us against 68.3, 128 columns
+// 101.9) and on two of three isothermal ones; 256 x 256 isothermal takes 47.0 us, 64 x 5 42.3.
 bool fp64_small_rows(int nx, int ny, int sms, int& rows) {
   auto tiles = [&](int cols, int r) {
     return (long long)((nx + tile_cols(cols) - 1) / tile_cols(cols)) * ((ny + r - 1) / r);
@@ -1187,7 +1191,8 @@ lbm_status lbm_autotune(lbm_ctx* c, int32_t trial_steps, int32_t* cols_out, int3
   if (!c || trial_steps < 1) return LBM_EINVAL;
   if (!c->have_params) return fail(c, LBM_ESTATE, "lbm_set_params first");
   DeviceGuard g(c->device);
-  static const int kCols[] = {64, 128, 256};
+  // first the default tiling, where that is not 128 columns with their default plan (fp64_small_rows)
+  static const int kCols[] = {0, 64, 128, 256};
   static const int kRows[] = {0, 4, 7, 10, 16, 24, 32, 48};
   cudaEvent_t e0, e1;
   LBM_CUDA(c, cudaEventCreate(&e0));
@@ -1200,7 +1205,7 @@ lbm_status lbm_autotune(lbm_ctx* c, int32_t trial_steps, int32_t* cols_out, int3
   lbm_status s = LBM_OK;
   for (int col : kCols) {
     for (int r : kRows) {
-      if (r > c->ny) continue;
+      if (r > c->ny || (col == 0 && (r > 0 || c->prec != LBM_FP64))) continue;
       if ((s = lbm_set_tiling(c, col, r)) != LBM_OK) break;
       if ((s = lbm_step_async(c, 2)) != LBM_OK) break;  // warm-up
       cudaEventRecord(e0, c->stream);
@@ -1224,7 +1229,9 @@ lbm_status lbm_autotune(lbm_ctx* c, int32_t trial_steps, int32_t* cols_out, int3
   cudaEventDestroy(e1);
   if (s != LBM_OK) return s;
   if ((s = lbm_set_tiling(c, best_c, best_r)) != LBM_OK) return s;
-  if (cols_out) *cols_out = best_c;
+  // the default tiling by what it is: 64 columns and uniform bands, or 128 and their default plan
+  if (best_c == 0 && c->cols != 128) best_r = c->plan.short_rows;
+  if (cols_out) *cols_out = c->cols;
   if (rows_out) *rows_out = best_r;
   return lbm_sync(c);
 }
