@@ -285,7 +285,9 @@ constexpr int kMinRows = 4;          // smallest band a step tiling may use
 constexpr int kMaxDim = 1 << 20;
 
 constexpr size_t kAlign = 256;
-constexpr int kMaxFlatTiles = 1368;  // FLAT_AUTO_ROUNDS tiles on each of three CTAs of 152 SMs
+// The SMs that a context's memory is laid out for (lbm_required_bytes names no device): on a GPU with
+// more, a lattice whose flat launch would take more tiles than reserved goes by the strip kernel.
+constexpr int kLayoutSms = 152;
 
 // Barrier status, totals and done counts of a flat launch, cleared together before it.
 size_t flat_state_bytes(int tiles) {
@@ -304,7 +306,8 @@ struct Layout {
       off_tiles_step, off_tiles_aux, off_flat, off_tiles_flat, total;
 };
 
-Layout make_layout(int nx, int ny, lbm_precision prec) {
+// flat: with room for the flat launch's tables (not for a batch's members: the batch has them).
+Layout make_layout(int nx, int ny, lbm_precision prec, bool flat = true) {
   Layout L{};
   const size_t elt = prec == LBM_FP64 ? 8 : 4;
   L.pitch = (nx + 31) / 32 * 32;
@@ -327,8 +330,8 @@ Layout make_layout(int nx, int ny, lbm_precision prec) {
   L.off_ring = off; off += align_up((size_t)RING * NDIAG * sizeof(double));
   L.off_tiles_step = off; off += align_up((size_t)L.max_tiles * sizeof(Tile));
   L.off_tiles_aux = off; off += align_up((size_t)L.max_tiles * sizeof(Tile));
-  L.max_flat = prec == LBM_FP32 ? (int)std::min<long long>(kMaxFlatTiles, L.max_tiles) : 0;
-  L.off_flat = off; off += align_up(flat_state_bytes(L.max_flat));
+  L.max_flat = prec == LBM_FP32 && flat ? flat_max_tiles(nx, ny, kLayoutSms, FLAT_AUTO_ROUNDS) : 0;
+  L.off_flat = off; off += L.max_flat ? align_up(flat_state_bytes(L.max_flat)) : 0;
   L.off_tiles_flat = off; off += align_up((size_t)L.max_flat * sizeof(FlatTile));
   L.total = off;
   return L;
@@ -662,7 +665,7 @@ void reset_state_mirror(lbm_ctx* c, long long step, int local, double rho_avg_pr
 }
 
 lbm_status create_impl(lbm_ctx** out, int32_t nx, int32_t ny, lbm_precision prec, int32_t device, void* stream,
-                       void* dev_buf, size_t dev_bytes) {
+                       void* dev_buf, size_t dev_bytes, bool member = false) {
   if (!out) return LBM_EINVAL;
   *out = nullptr;
   if (nx < 1 || ny < 1 || nx > kMaxDim || ny > kMaxDim) return LBM_EINVAL;
@@ -676,7 +679,8 @@ lbm_status create_impl(lbm_ctx** out, int32_t nx, int32_t ny, lbm_precision prec
   c->ny = ny;
   c->prec = prec;
   c->device = device;
-  c->L = make_layout(nx, ny, prec);
+  c->member = member;
+  c->L = make_layout(nx, ny, prec, !member);
   DeviceGuard g(device);
   cudaError_t e = cudaSetDevice(device);
   if (e != cudaSuccess) { delete c; return LBM_ECUDA; }
@@ -740,7 +744,10 @@ lbm_status create_impl(lbm_ctx** out, int32_t nx, int32_t ny, lbm_precision prec
 namespace pplbm {
 Inst lbm_internal_inst(const lbm_ctx* c) { return c->hinst; }
 unsigned long long lbm_internal_params_gen(const lbm_ctx* c) { return c->params_gen; }
-void lbm_internal_set_member(lbm_ctx* c) { c->member = true; }
+lbm_status lbm_internal_create_member(lbm_ctx** out, int32_t nx, int32_t ny, lbm_precision prec, int32_t device,
+                                      void* stream) {
+  return create_impl(out, nx, ny, prec, device, stream, nullptr, 0, true);
+}
 }  // namespace pplbm
 
 extern "C" {

@@ -396,9 +396,8 @@ lbm_status lbm_batch_add(lbm_batch* b, int32_t nx, int32_t ny, const lbm_params*
   if (!b || !slot) return LBM_EINVAL;
   if (!p || p->thermal != b->thermal) return bfail(b, LBM_EINVAL, "member must match the batch's thermal flag");
   lbm_ctx* c = nullptr;
-  lbm_status s = lbm_create(&c, nx, ny, b->prec, b->device, b->stream);
+  lbm_status s = lbm_internal_create_member(&c, nx, ny, b->prec, b->device, b->stream);
   if (s != LBM_OK) return bfail(b, s, "member creation failed");
-  lbm_internal_set_member(c);
   s = lbm_set_params(c, p);
   if (s != LBM_OK) {
     b->err = lbm_last_error(c);

@@ -134,4 +134,15 @@ int flat_rows(const std::vector<FlatSize>& sizes, int sms, int max_rounds, const
   return best;
 }
 
+int flat_max_tiles(int nx, int ny, int sms, int max_rounds) {
+  const int w = flat_width(nx), strips = (nx + w - 1) / w;
+  long long most = 0;
+  for (int rows = 4; rows <= FLAT_MAX_ROWS; ++rows) {
+    const long long tiles = (long long)strips * ((ny + rows - 1) / rows);
+    const int per_sm = 4 * (16384 / (FLAT_REGS * 32)) / (rows + 6);  // CTAs that the four register files hold
+    if (tiles <= (long long)max_rounds * per_sm * sms) most = std::max(most, tiles);
+  }
+  return (int)most;
+}
+
 }  // namespace pplbm

@@ -364,6 +364,9 @@ struct FlatSize {
 bool build_flat_tiles(int inst, int nx, int ny, int geometry, int rows, std::vector<FlatTile>& out);
 // per_sm_by_warps: resident CTAs per SM by warps per CTA (indices 0 .. 21).
 int flat_rows(const std::vector<FlatSize>& sizes, int sms, int max_rounds, const int* per_sm_by_warps);
+// The most tiles that a lattice's flat launch takes on `sms` SMs with at most max_rounds tiles a CTA; 0
+// where it is too large for it at every tile height.
+int flat_max_tiles(int nx, int ny, int sms, int max_rounds);
 constexpr int FLAT_MAX_STEPS = 1 << 27;  // of a launch: steps times rows stay below 2^32
 constexpr double FLAT_ROUND_COST = 10.0;  // in warps
 // Rounds (tiles per CTA) up to which the flat launch is taken.  A round costs about 6 us whatever the
@@ -470,7 +473,8 @@ int resident_ctas_f64(int thermal, int cols, int kernel);
 Inst lbm_internal_inst(const lbm_ctx* c);
 // Changes whenever the context's descriptor is rewritten (parameters or a loaded state).
 unsigned long long lbm_internal_params_gen(const lbm_ctx* c);
-// Marks a context as a batch's member (before its parameters are set).
-void lbm_internal_set_member(lbm_ctx* c);
+// A context for a batch's member: as lbm_create, without a flat launch of its own.
+lbm_status lbm_internal_create_member(lbm_ctx** out, int32_t nx, int32_t ny, lbm_precision prec, int32_t device,
+                                      void* stream);
 
 }  // namespace pplbm
