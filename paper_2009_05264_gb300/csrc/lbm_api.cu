@@ -515,10 +515,10 @@ int step_kernel(const lbm_ctx* c, int cols) {
 lbm_status plan_flat(lbm_ctx* c) {
   c->flat_tiles = 0;
   if (c->member || !c->have_params || !c->rows_default || c->cols != 128 || step_kernel(c, c->cols) != FORM_STRIP) return LBM_OK;
-  int dev = 0, sms = 0, per_sm[22] = {};
+  int dev = 0, sms = 0, per_sm[21] = {};
   LBM_CUDA(c, cudaGetDevice(&dev));
   LBM_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  for (int w = 10; w <= 21; ++w) per_sm[w] = flat_resident_ctas(c->thermal, step_flags(c->hinst), true, w);
+  for (int w = 10; w <= 20; ++w) per_sm[w] = flat_resident_ctas(c->thermal, step_flags(c->hinst), true, w);
   const int rows = flat_rows({{c->nx, c->ny}}, sms, FLAT_AUTO_ROUNDS, per_sm);
   if (rows == 0) return LBM_OK;
   std::vector<FlatTile> t;

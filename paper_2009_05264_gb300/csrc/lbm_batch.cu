@@ -108,10 +108,10 @@ size_t flat_state_bytes(size_t insts, size_t tiles) {
 lbm_status plan_flat(lbm_batch* b, const std::vector<Inst>& insts) {
   b->flat_tiles = 0;
   if (insts.empty() || b->launch_kernel != FORM_STRIP || b->rows != 0 || b->cols != 128) return LBM_OK;
-  int dev = 0, sms = 0, per_sm[22] = {};
+  int dev = 0, sms = 0, per_sm[21] = {};
   LBM_BCUDA(b, cudaGetDevice(&dev));
   LBM_BCUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  for (int w = 10; w <= 21; ++w) per_sm[w] = flat_resident_ctas(b->thermal, b->flags, false, w);
+  for (int w = 10; w <= 20; ++w) per_sm[w] = flat_resident_ctas(b->thermal, b->flags, false, w);
   std::vector<FlatSize> sizes;
   for (const Inst& I : insts) sizes.push_back({I.nx, I.ny});
   const int rows = flat_rows(sizes, sms, FLAT_BATCH_ROUNDS, per_sm);

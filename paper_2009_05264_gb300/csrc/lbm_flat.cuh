@@ -8,8 +8,8 @@
 //
 // Why: a small lattice's step is a chain of latencies, not of work.  Marching eight rows (four and
 // the halo) in one warp costs eight dependent passes of about 600 instructions at six cycles each,
-// 16 us of a 21 us step on 1000 x 100; here the chain is one row's, and a tile of up to 15 rows
-// recomputes 4 of its 19 rows instead of 4 of 8.  Measured per step: 1000 x 100 channel 6.7 us
+// 16 us of a 21 us step on 1000 x 100; here the chain is one row's, and a tile of up to 14 rows
+// recomputes 4 of its 18 rows instead of 4 of 8.  Measured per step: 1000 x 100 channel 6.7 us
 // (strip kernel 20.5, the one-column kernel before it 23), 600 x 80 5.3 us (28 before), 251 x 190
 // periodic 5.0 us (23 before), 100 x 50 isothermal 3.5 us.  What is left on 1000 x 100 (cycles at
 // 2.07 GHz, one tile's trace): 1300 until the tiles around are seen done, 2000 to 3000 for 92 KB of
@@ -32,11 +32,12 @@
 
 namespace pplbm {
 
-constexpr int FLAT_MAX_ROWS = 15;                  // output rows per tile
+constexpr int FLAT_MAX_ROWS = 14;                  // output rows per tile
 constexpr int FLAT_MAX_WARPS = FLAT_MAX_ROWS + 6;  // with the halo rows' warps and the two without a row
 constexpr int FLAT_WIDTH = 60;                     // output columns per tile, at most
 constexpr int FLAT_MAX_ROUNDS = 8;                  // tiles per CTA, at most
-// Registers per thread: 21 warps of one CTA, or two CTAs of 10, fill the register file of an SM.
+// Registers per thread: 20 warps, one CTA of 14 rows or two of 4, fill the register files of an SM
+// (five warps of 96 registers in each quarter's 16384).
 constexpr int FLAT_REGS = 96;
 
 // Shared memory per row: psi (the pair, east minus west, east plus west) and u_act,y; density and

@@ -362,7 +362,7 @@ struct FlatSize {
   int nx, ny;
 };
 bool build_flat_tiles(int inst, int nx, int ny, int geometry, int rows, std::vector<FlatTile>& out);
-// per_sm_by_warps: resident CTAs per SM by warps per CTA (indices 0 .. 21).
+// per_sm_by_warps: resident CTAs per SM by warps per CTA (indices 0 .. 20).
 int flat_rows(const std::vector<FlatSize>& sizes, int sms, int max_rounds, const int* per_sm_by_warps);
 // The most tiles that a lattice's flat launch takes on `sms` SMs with at most max_rounds tiles a CTA; 0
 // where it is too large for it at every tile height.

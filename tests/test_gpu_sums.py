@@ -3,7 +3,7 @@
 The first step's record is formed from the initialised populations as they are, so its mass, energy and
 heater-row temperature are known: each node's density and temperature deviations are FP32 sums of its
 populations in the kernels' order, and their totals are exact sums of those (math.fsum).  The flat launch
-sums up to 15 rows of a column in FP32 with the errors carried along (a relative error of about 2^-47 of
+sums up to 14 rows of a column in FP32 with the errors carried along (a relative error of about 2^-47 of
 the magnitudes summed) and rounds each tile's sums to the fixed-point totals (52 - ceil(log2 m) fraction
 bits, m the nodes that feed a total); the heater row enters FP64 node by node in every loop.
 """
