@@ -103,8 +103,25 @@ size_t flat_state_bytes(size_t insts, size_t tiles) {
   return kFlatHead + insts * sizeof(FlatState) + tiles * FLAT_DONE_STRIDE * sizeof(unsigned);
 }
 
+// Room for count elements (`bytes` bytes) at *p, of capacity *cap; false: there is none, and *p is null.
+template <typename T>
+bool flat_reserve(T** p, size_t* cap, size_t count, size_t bytes) {
+  if (count <= *cap) return true;
+  if (*p) cudaFree(*p);
+  *p = nullptr;
+  *cap = 0;
+  if (cudaMalloc(p, bytes) != cudaSuccess) {
+    *p = nullptr;
+    cudaGetLastError();  // not an error of the launches to come
+    return false;
+  }
+  *cap = count;
+  return true;
+}
+
 // The flat launch's tiles over all members, where the strip kernel runs with the default tiling and
-// the members together are small enough (FLAT_BATCH_ROUNDS).
+// the members together are small enough (FLAT_BATCH_ROUNDS).  Without memory for its tables the batch
+// steps by the strip kernel, which needs none.
 lbm_status plan_flat(lbm_batch* b, const std::vector<Inst>& insts) {
   b->flat_tiles = 0;
   if (insts.empty() || b->launch_kernel != FORM_STRIP || b->rows != 0 || b->cols != 128) return LBM_OK;
@@ -119,22 +136,10 @@ lbm_status plan_flat(lbm_batch* b, const std::vector<Inst>& insts) {
   std::vector<FlatTile> t;
   for (size_t i = 0; i < insts.size(); ++i)
     if (!build_flat_tiles((int)i, insts[i].nx, insts[i].ny, insts[i].geometry, rows, t)) return LBM_OK;
-  if (t.size() > b->cap_flat) {
-    if (b->d_flat_tiles) cudaFree(b->d_flat_tiles);
-    b->d_flat_tiles = nullptr;
-    b->cap_flat = 0;
-    if (cudaMalloc(&b->d_flat_tiles, t.size() * sizeof(FlatTile)) != cudaSuccess)
-      return bfail(b, LBM_ENOMEM, "flat tile table");
-    b->cap_flat = t.size();
-  }
   const size_t bytes = flat_state_bytes(insts.size(), t.size());
-  if (bytes > b->cap_flat_state) {
-    if (b->d_flat_state) cudaFree(b->d_flat_state);
-    b->d_flat_state = nullptr;
-    b->cap_flat_state = 0;
-    if (cudaMalloc(&b->d_flat_state, bytes) != cudaSuccess) return bfail(b, LBM_ENOMEM, "flat launch state");
-    b->cap_flat_state = bytes;
-  }
+  if (!flat_reserve(&b->d_flat_tiles, &b->cap_flat, t.size(), t.size() * sizeof(FlatTile)) ||
+      !flat_reserve(&b->d_flat_state, &b->cap_flat_state, bytes, bytes))
+    return LBM_OK;
   LBM_BCUDA(b, cudaMemcpyAsync(b->d_flat_tiles, t.data(), t.size() * sizeof(FlatTile), cudaMemcpyHostToDevice, b->stream));
   LBM_BCUDA(b, cudaStreamSynchronize(b->stream));
   b->flat_tiles = (int)t.size();

@@ -123,7 +123,7 @@ extern "C" lbm_status lbm_step_noalloc(const lbm_params* p, int32_t nx, int32_t 
   fill_tiles_kernel<<<(ntiles + 255) / 256, 256, 0, s>>>(tiles, nx, ny, w, rows, strips, ntiles);
   if (cudaGetLastError() != cudaSuccess) return LBM_ECUDA;
   // The caller's buffers are dense (pitch nx, any nx) and only element-aligned, so the
-  // paired kernel's 8-byte accesses are not valid here: always the one-column form.
+  // strip kernel's 8-byte accesses are not valid here: always the one-column form.
   if (launch_lbm(prec == LBM_FP64, p->thermal, kNoAllocCols, MODE_STEP, LBM_KERNEL_SCALAR, step_flags(I),
                  reinterpret_cast<const Inst*>(base + kOffInst), tiles, ntiles, s) != cudaSuccess)
     return LBM_ECUDA;
