@@ -311,11 +311,12 @@ __device__ __forceinline__ bool flat_serve(const Inst& I, const StripTile& t, co
   const float2* const sM = smem + lane + 32 * nrows * (4 + 2 * (turn & 1));
   const float2* const sE = sM + 32 * nrows;
   const bool out_a = lane >= 1 && lane <= t.wout / 2 && t.xs + 2 * lane < t.nx, out_b = out_a && t.xs + 2 * lane + 1 < t.nx;
-  // A lane's two columns over the tile's rows: FP32 sums with their rounding errors summed beside them
-  // (Knuth's two-sum), about 48 bits in all.  (An FP64 addition takes the warp 64 cycles.)  Every tile
-  // waits for the mass, so the rows' loads are issued together, the loop unrolled for the most rows:
-  // 1000 x 100 7.74 us a step within a call against 7.85 unrolled by 4, 600 x 80 7.6 against 8.0; FP32
-  // sums alone 7.64 and 7.9.
+  // A lane's two columns over the tile's rows: four rows at a time in FP32 (the lowest bands of the
+  // other kernels), those sums with their rounding errors summed beside them (Knuth's two-sum), about
+  // 48 bits in all.  An FP64 addition takes the warp 64 cycles, and every instruction here waits among
+  // the rows' warps on the way to the mass that every tile waits for: 1000 x 100 6.62 us a step, 1500 x
+  // 150 13.0, 600 x 80 with bubbles 5.74; with the errors of every row 6.82, 13.5 and 5.84, and rolled
+  // loops of four or seven rows 7.3 to 7.5, 15.2 and 6.7.
   auto pair_sum = [&](float2 s, float2 c) {
     if (!out_a) s.x = c.x = 0.0f;
     if (!out_b) s.y = c.y = 0.0f;
@@ -325,13 +326,20 @@ __device__ __forceinline__ bool flat_serve(const Inst& I, const StripTile& t, co
   };
   auto column_sum = [&](const float2* v) {
     float2 s = make_float2(0.0f, 0.0f), c = s;
+    float2 a = s;
+    auto take = [&] {
+      const float2 h = v_add(s, a), z = v_sub(h, s);
+      c = v_add(c, v_add(v_sub(s, v_sub(h, z)), v_sub(a, z)));
+      s = h;
+    };
 #pragma unroll
     for (int w = 0; w < FLAT_MAX_ROWS; ++w) {
       if (w >= rows) break;
-      const float2 a = v[(w + 2) * 32], h = v_add(s, a), z = v_sub(h, s);
-      c = v_add(c, v_add(v_sub(s, v_sub(h, z)), v_sub(a, z)));
-      s = h;
+      a = w % 4 == 0 ? v[(w + 2) * 32] : v_add(a, v[(w + 2) * 32]);
+      if (w == 3) s = a;
+      else if (w % 4 == 3) take();
     }
+    if (rows % 4 != 0) take();
     return pair_sum(s, c);
   };
   const double scale = I.fix_scale[lane < NPART ? lane : 0];

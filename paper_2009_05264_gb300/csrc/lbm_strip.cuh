@@ -58,9 +58,9 @@ struct StripParams {
 
 // Per-lane sums of a tile (output nodes only: the caller drops the other lanes' at the end).
 struct StripSums {
-  float2 m, e, h;
+  float2 m, e;
+  double h, open;
   float fi, fo, va, wv, hv, zv;
-  double open;
   bool bad;
 };
 
@@ -114,7 +114,10 @@ __device__ __forceinline__ void strip_rows(const Inst& I, const StripTile& t, fl
         S.m = v_add(S.m, n.drho);
         if (THERMAL) {
           S.e = v_add(S.e, n.dT);
-          if (lo) S.h = L.heater_dT(n.dT);
+          if (lo) {
+            const float2 h = L.heater_dT(n.dT);
+            S.h = (double)h.x + (double)h.y;
+          }
         }
         if (L.bubbles) {
           const int hx = I.heater_x0, hl = I.heater_len;
@@ -258,7 +261,7 @@ __device__ __forceinline__ void strip_tile(const Inst* __restrict__ insts, const
       strip_rows<THERMAL, FULL, true>(I, t, rra, step, ring, S);
   }
   if (S.bad) atomicOr(&st->status, STATUS_UNSTABLE);
-  const double acc[NPART] = {(double)S.m.x + (double)S.m.y, (double)S.e.x + (double)S.e.y, (double)S.h.x + (double)S.h.y,
+  const double acc[NPART] = {(double)S.m.x + (double)S.m.y, (double)S.e.x + (double)S.e.y, S.h,
                              (double)S.fi, (double)S.fo, (double)S.va, (double)S.wv, (double)S.hv, (double)S.zv};
   if (!FULL && tile.interior)
     post_partials<STRIP_MAX_WARPS, THERMAL, MODE_STEP, 3>(I, st, tile, acc, sh.red, &sh.last, step);

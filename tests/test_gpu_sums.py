@@ -2,10 +2,11 @@
 
 The first step's record is formed from the initialised populations as they are, so its mass, energy and
 heater-row temperature are known: each node's density and temperature deviations are FP32 sums of its
-populations in the kernels' order, and their totals are exact sums of those (math.fsum).  The flat launch
-sums up to 14 rows of a column in FP32 with the errors carried along (a relative error of about 2^-47 of
-the magnitudes summed) and rounds each tile's sums to the fixed-point totals (52 - ceil(log2 m) fraction
-bits, m the nodes that feed a total); the heater row enters FP64 node by node in every loop.
+populations in the kernels' order.  The flat launch sums a column's rows four at a time in FP32, from the
+bottom of each band, and those sums with the errors carried along (a relative error of about 2^-47 of the
+magnitudes summed), and rounds each tile's sums to the fixed-point totals (52 - ceil(log2 m) fraction
+bits, m the nodes that feed a total): the totals are exact sums (math.fsum) of the FP32 sums of four rows.
+The heater row enters FP64 node by node in every loop.
 """
 import math
 
@@ -25,10 +26,25 @@ def grid(tiles, m):
     return tiles * 2.0 ** -(52 - math.ceil(math.log2(m)) + 1)
 
 
-@pytest.mark.parametrize("nx,ny,geometry,loop", [
-    (1000, 100, "channel", "auto"), (599, 80, "walls", "auto"), (1500, 150, "channel", "auto"), (61, 5, "pool", "auto"),
-    (1000, 100, "channel", "launches"), (3000, 300, "walls", "auto")])
-def test_first_record_is_the_exact_sum(nx, ny, geometry, loop):
+def fours(v, bands):
+    """FP32 sums of four rows of a column at a time, from the bottom of each of `bands` bands."""
+    ny, out = len(v), []
+    start = [b * ny // bands for b in range(bands + 1)]
+    for y0, y1 in zip(start, start[1:]):
+        for y in range(y0, y1, 4):
+            a = v[y]
+            for row in v[y + 1:min(y + 4, y1)]:
+                a = a + row
+            out.append(a)
+    assert out[0].dtype == np.float32
+    return np.array(out, dtype=np.float64)
+
+
+# bands: of the flat launch's tiles (13, 6, 13 and 4 rows), None where another kernel runs
+@pytest.mark.parametrize("nx,ny,geometry,loop,bands", [
+    (1000, 100, "channel", "auto", 8), (599, 80, "walls", "auto", 14), (1500, 150, "channel", "auto", 12),
+    (61, 5, "pool", "auto", 2), (1000, 100, "channel", "launches", None), (3000, 300, "walls", "auto", None)])
+def test_first_record_is_the_exact_sum(nx, ny, geometry, loop, bands):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2009_05264_gb300 import lbm as L
@@ -43,7 +59,7 @@ def test_first_record_is_the_exact_sum(nx, ny, geometry, loop):
     lat = L.Lattice(nx, ny, "fp32")
     lat.set_params(p)
     lat.set_step_loop(loop)
-    flat = loop == "auto" and nx * ny < 300000
+    assert (lat.step_form == "flat") == (bands is not None)
     lat.init_fields(rho, np.zeros_like(rho), np.zeros_like(rho), T)
     f, g = lat.populations()
     rho_ref = p["rho_out"] if geometry == "channel" else p["init_rho_out"]
@@ -55,10 +71,11 @@ def test_first_record_is_the_exact_sum(nx, ny, geometry, loop):
     lat.step(1)
     d = lat.diagnostics()
     n, tiles = nx * ny, -(-nx // 56) * -(-ny // 4)
-    if flat:
-        mass, energy = (math.fsum(v.astype(np.float64).ravel()) for v in (drho, dT))
-        for got, want, ref, v in ((d["mass"], mass, rho_ref, drho), (d["energy"], energy, T_ref, dT)):
-            assert abs(got - (want + n * ref)) <= grid(tiles, n) + 2.0 ** -47 * float(np.abs(v).sum()) + 1e-15 * n * ref
+    if bands:
+        for got, v, ref in ((d["mass"], drho, rho_ref), (d["energy"], dT, T_ref)):
+            sums = fours(v, bands)
+            want = math.fsum(sums.ravel()) + n * ref
+            assert abs(got - want) <= grid(tiles, n) + 2.0 ** -47 * float(np.abs(sums).sum()) + 1e-15 * n * ref
     heat = math.fsum(dT[0, hx:hx + hl].astype(np.float64))
     T_heat = (p["Tin_R"] + p["dTheat_R"]) * Tc
     want = (T_heat - (heat / hl + T_ref)) / (T_heat - d["energy"] / n)
