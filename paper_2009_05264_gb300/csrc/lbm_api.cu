@@ -306,8 +306,7 @@ struct Layout {
       off_tiles_step, off_tiles_aux, off_flat, off_tiles_flat, total;
 };
 
-// flat: with room for the flat launch's tables (not for a batch's members: the batch has them).
-Layout make_layout(int nx, int ny, lbm_precision prec, bool flat = true) {
+Layout make_layout(int nx, int ny, lbm_precision prec) {
   Layout L{};
   const size_t elt = prec == LBM_FP64 ? 8 : 4;
   L.pitch = (nx + 31) / 32 * 32;
@@ -330,7 +329,7 @@ Layout make_layout(int nx, int ny, lbm_precision prec, bool flat = true) {
   L.off_ring = off; off += align_up((size_t)RING * NDIAG * sizeof(double));
   L.off_tiles_step = off; off += align_up((size_t)L.max_tiles * sizeof(Tile));
   L.off_tiles_aux = off; off += align_up((size_t)L.max_tiles * sizeof(Tile));
-  L.max_flat = prec == LBM_FP32 && flat ? flat_max_tiles(nx, ny, kLayoutSms, FLAT_AUTO_ROUNDS) : 0;
+  L.max_flat = prec == LBM_FP32 ? flat_max_tiles(nx, ny, kLayoutSms, FLAT_AUTO_ROUNDS) : 0;
   L.off_flat = off; off += L.max_flat ? align_up(flat_state_bytes(L.max_flat)) : 0;
   L.off_tiles_flat = off; off += align_up((size_t)L.max_flat * sizeof(FlatTile));
   L.total = off;
@@ -680,7 +679,7 @@ lbm_status create_impl(lbm_ctx** out, int32_t nx, int32_t ny, lbm_precision prec
   c->prec = prec;
   c->device = device;
   c->member = member;
-  c->L = make_layout(nx, ny, prec, !member);
+  c->L = make_layout(nx, ny, prec);
   DeviceGuard g(device);
   cudaError_t e = cudaSetDevice(device);
   if (e != cudaSuccess) { delete c; return LBM_ECUDA; }
