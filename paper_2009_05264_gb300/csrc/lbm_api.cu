@@ -606,8 +606,8 @@ bool overlapped(lbm_ctx* c) {
 // step tiling is one wave of the persistent kernel, where a step's launch gap and kernel
 // boundary are a large part of it, or at least two and a half waves that the overlapped form
 // can run (the end of each step then overlaps the start of the next; with fewer tiles per CTA
-// the next step's first tiles mostly wait, and one launch per step measured faster).  Only
-// the one-column kernel (general or interior path) has a persistent form.
+// the next step's first tiles mostly wait, and one launch per step measured faster).  All
+// kernels but the TMA form have a persistent form.
 bool use_persistent(lbm_ctx* c) {
   if (c->loop == LBM_LOOP_LAUNCHES) return false;
   const int kernel = step_kernel(c, c->cols);

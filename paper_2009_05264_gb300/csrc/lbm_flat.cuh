@@ -9,9 +9,9 @@
 // Why: a small lattice's step is a chain of latencies, not of work.  Marching eight rows (four and
 // the halo) in one warp costs eight dependent passes of about 600 instructions at six cycles each,
 // 16 us of a 21 us step on 1000 x 100; here the chain is one row's, and a tile of up to 14 rows
-// recomputes 4 of its 18 rows instead of 4 of 8.  Measured per step: 1000 x 100 channel 6.7 us
-// (strip kernel 20.5, the one-column kernel before it 23), 600 x 80 5.3 us (28 before), 251 x 190
-// periodic 5.0 us (23 before), 100 x 50 isothermal 3.5 us.  What is left on 1000 x 100 (cycles at
+// recomputes 4 of its 18 rows instead of 4 of 8.  Measured per step: 1000 x 100 channel 6.6 us
+// (strip kernel 18.5 at its best tiling, the one-column kernel before it 23), 600 x 80 5.4 us (17.8;
+// 28), with bubbles 5.8, 251 x 190 periodic 5.2 us (19.0; 23), 100 x 50 5.0 us, isothermal 3.8.  What is left on 1000 x 100 (cycles at
 // 2.07 GHz, one tile's trace): 1300 until the tiles around are seen done, 2000 to 3000 for 92 KB of
 // populations from L2, 1300 for phase A, 1500 for B, 700 for C, 1200 until the stores are counted.
 //

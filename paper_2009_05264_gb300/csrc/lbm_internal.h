@@ -370,10 +370,11 @@ int flat_max_tiles(int nx, int ny, int sms, int max_rounds);
 constexpr int FLAT_MAX_STEPS = 1 << 27;  // of a launch: steps times rows stay below 2^32
 constexpr double FLAT_ROUND_COST = 10.0;  // in warps
 // Rounds (tiles per CTA) up to which the flat launch is taken.  A round costs about 6 us whatever the
-// size, the strip kernel no less than 20 us a step: 1500 x 150 (2 rounds) 12.7 against 20.1 us,
-// 1800 x 160 (3) 17.0 against 19.9, 2000 x 200 (4) 24.2 against 24.6, 2500 x 220 (5) 31.3 against
-// 26.7.  A batch's strip kernel reads its constants from shared memory and is a little slower:
-// four 128 x 512 pools (3 rounds) 21.5 against 28.9 us, six (5) 34.1 against 31.8.
+// size, the strip kernel no less than 18 us a step: 1500 x 150 (2 rounds) 13.1 us against 21.2 (the
+// best of five strip tilings and loops), 1800 x 160 (3) 18.2 against 21.2; with the limit raised, 2000
+// x 200 (4) 24.2 against 24.6, 2500 x 220 (5) 31.3 against 26.7.  A batch's strip kernel reads its
+// constants from shared memory and is a little slower: three 128 x 512 pools 19.0 against 26.6 us,
+// four 21.3 against 29.1, five (4 rounds) 27.8 against 30.9, six (5) 34.1 against 31.8.
 constexpr int FLAT_AUTO_ROUNDS = 3, FLAT_BATCH_ROUNDS = 4;
 // nsteps steps of the step kernel in one cooperative launch (tiles drawn dynamically from a
 // counter, a bounded grid barrier between steps; MODE_STEP only).  grid <= resident CTAs of

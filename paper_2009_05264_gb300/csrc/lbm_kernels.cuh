@@ -22,8 +22,9 @@
 // outputs plus two halo columns per side (the last 4 lanes idle, so every CTA's
 // output starts on a 32-byte sector).  The force at a node needs psi on its 8
 // neighbours and the divergence of u_act in the g source needs u_act (hence the
-// force) on the 4 neighbours, so psi is needed two nodes out: the CTA keeps
-// three-row rings of psi and u_act in shared memory.  At iteration k it pulls
+// force) on the 4 neighbours, so psi is needed two nodes out: the CTA keeps a
+// row of psi (each thread what it needs of the two rows below in registers) and a
+// three-row ring of u_act in shared memory.  At iteration k it pulls
 // row r = y0 - 2 + k (phase A: boundary fill, moments, EOS), computes force, u_act
 // and the f collision of row r - 1 (phase B) and the g collision of row r - 2
 // (phase C), with a barrier after A and after B.  Each thread's pulled

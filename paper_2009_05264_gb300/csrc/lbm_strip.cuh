@@ -14,12 +14,13 @@
 // Why this shape: the one-column kernel's step took 20.9 warp-instructions per node, two
 // barriers per row and 18 four-byte asynchronous copies per node, and was bound by their
 // latency at four warps per scheduler with neither DRAM nor any pipe busy.  Two nodes per lane
-// halve the instructions of everything (12.1 warp-instructions per node), the shuffles replace the
+// halve the instructions of everything (13.2 warp-instructions per node in the overlapped loop, its
+// waits included), the shuffles replace the
 // shared-memory rings of psi and u_act, and without barriers the loads of row r + 1, issued
 // between phases A and B into registers, have the rest of the iteration to arrive.  A warp loses
-// 4 of its 64 columns to the halo, as much as a 128-column CTA did.  8000 x 800 channel: 175 us a
-// step (36.5 GLUPS, 152 B of DRAM traffic a node = 0.82 of the copy rate) against 196; issue
-// active 37 %, the warps mostly wait for their loads.  Tried and slower: the rows staged in shared
+// 4 of its 64 columns to the halo, as much as a 128-column CTA did.  8000 x 800 channel: 172 to
+// 176 us a step (36.4 to 37.2 GLUPS; 156 B of DRAM traffic a node, 5.7 TB/s = 0.84 of the copy
+// rate) against 196; issue active 28 %, the warps mostly wait for their loads.  Tried and slower: the rows staged in shared
 // memory by 16-byte cp.async (204 us), the loop unrolled by 2 or 3 (194, 254: spills),
 // 144 registers for 14 warps per SM (283, spills), 184 for 10 (197).
 //
