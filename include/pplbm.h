@@ -179,7 +179,7 @@ lbm_status lbm_init_fields(lbm_ctx* ctx, const double* rho, const double* ux, co
                            const double* T, size_t n);
 
 /* Advance nsteps time steps (Eqs. 1-19 and the Sec. 2.C boundary conditions),
- * fused into one kernel per step, then wait and return the stability status.
+ * fused into one kernel (a launch per step or per call, lbm_set_step_loop), then wait and return the stability status.
  * Errors: LBM_ESTATE (no params), LBM_EUNSTABLE, LBM_ECUDA. */
 lbm_status lbm_step(lbm_ctx* ctx, int64_t nsteps);
 
